@@ -237,9 +237,9 @@ dg_status dg_operator_set_face_pairs(dg_op* op, int32_t enable);
  * to the operator, or remove it (src = NULL).  Later dg_rhs, dg_step,
  * dg_solve, dg_step_host, dg_step_host_jobs and dg_step_static calls add
  * s(t) w to the Ez right-hand side of the element that contains the point:
- * after each stage launch one small kernel adds dt s(t) w to that element's
- * residual and b_i dt s(t) w to its fields (t: the stage time t0 + (n + c_i)
- * dt), which is the stage update with the source in the right-hand side.
+ * each stage launch adds dt s(t) w to that element's residual and b_i dt
+ * s(t) w to its fields (t: the stage time t0 + (n + c_i) dt), which is the
+ * stage update with the source in the right-hand side.
  * The projected load w is computed on the host in FP64 and uploaded once
  * (an allocation of Np values, made here, not by the stepping calls).
  * Batches and servers take their own sources and ignore this one;

@@ -417,71 +417,60 @@ dg_status check_field(const dg_op* op, const void* p, const char* name, const ch
   return DG_OK;
 }
 
-// Ricker point source of an operator (dg_operator_set_source), applied after
-// a stage launch: the source element's Ez residual gains dt s(t) w and its
-// Ez values b times that.  This is the LSRK stage update with s(t) w added
-// to the right-hand side of Eq. dg-strong-explicit (w = M^-1 l(x_s) / J_k,
-// the projected point load).  rhs_only: q is a right-hand side, which gains
-// s(t) w.  s(t) = A (1 - 2 a^2) exp(-a^2), a = pi f (t - t0).
+// Ricker point source of an operator (dg_operator_set_source) at time t, for
+// the stage launch that takes `a`: dEz/dt of the source element gains s(t) w
+// (w = M^-1 l(x_s) / J_k, the projected point load), so its Ez residual
+// gains dt s(t) w and its Ez values b times that; s(t) = A (1 - 2 x^2)
+// exp(-x^2), x = pi f (t - t0).  dt = 1 for a right-hand side.  Nothing
+// without a source.  (A kernel of its own after every stage launch, the
+// earlier form, cost as much again as the stage on small meshes.)
 template <typename T>
-__global__ void point_source_kernel(T* q, T* res, const T* w, int Np, double t, double pif,
-                                    double t0, double amp, double dt, double b, int rhs_only) {
-  const int n = threadIdx.x;
-  if (n >= Np) return;
-  const double a = (t - t0) * pif;
-  const double s = amp * (1.0 - 2.0 * a * a) * exp(-a * a);
-  if (rhs_only) {
-    q[n] += static_cast<T>(s) * w[n];
-    return;
-  }
-  const T v = static_cast<T>(dt * s) * w[n];
-  res[n] += v;
-  q[n] += static_cast<T>(b) * v;
+void set_source(const dg_op* op, dgw::StageArgs<T>& a, double t, double dt) {
+  if (!op->has_src) return;
+  const double x = (t - op->src.t0) * (M_PI * op->src.f);
+  a.psrc_k = static_cast<int>(op->src_k);
+  a.psrc_w = static_cast<const T*>(op->d_src_w);
+  a.psrc_amp = static_cast<T>(dt * (op->src.amplitude * (1.0 - 2.0 * x * x) * std::exp(-x * x)));
 }
 
-// The point source after stage i of a step that starts at t (stage time
-// t + c_i dt), on the stage's output fields q and residual res; nothing
-// without a source.
+// nsteps LSRK steps ping-ponging between q and tmp (no copy back); returns
+// the buffer that holds the result
 template <typename T>
-cudaError_t stage_source(const dg_op* op, T* q, T* res, double t, double dt, int i,
-                         cudaStream_t s) {
-  if (!op->has_src) return cudaSuccess;
-  const int64_t off = 2 * op->fstride + op->src_k * op->Np;
-  point_source_kernel<T><<<1, 64, 0, s>>>(q + off, res + off, static_cast<const T*>(op->d_src_w),
-                                          op->Np, t + op->lsrk_c[i] * dt, M_PI * op->src.f,
-                                          op->src.t0, op->src.amplitude, dt, op->lsrk_b[i], 0);
-  op->launches.fetch_add(1, std::memory_order_relaxed);
-  return cudaGetLastError();
-}
-
-template <typename T>
-dg_status run_steps(const dg_op* op, T* q, T* res, double t0, double dt, int32_t nsteps,
-                    cudaStream_t s) {
+dg_status run_stages(const dg_op* op, T* q, T* tmp, T* res, double t0, double dt, int32_t nsteps,
+                     cudaStream_t s, T** result, const char* where) {
   dgw::StageArgs<T> a = base_args<T>(op);
   a.res = res;
   a.dt = static_cast<T>(dt);
   T* cur = q;
-  T* other = static_cast<T*>(op->d_qtmp);
+  T* other = tmp;
   for (int32_t n = 0; n < nsteps; ++n) {
     for (int i = 0; i < 5; ++i) {
       a.qin = cur;
       a.qout = other;
       a.a = static_cast<T>(op->lsrk_a[i]);
       a.b = static_cast<T>(op->lsrk_b[i]);
+      set_source<T>(op, a, t0 + n * dt + op->lsrk_c[i] * dt, dt);
       const int mode = (i == 0) ? dgw::kModeFirstStage : dgw::kModeStage;
       cudaError_t err = launch_order<T>(op, a, mode, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_step: kernel launch");
+      if (err != cudaSuccess) return cuda_fail(err, where);
       op->launches.fetch_add(1, std::memory_order_relaxed);
-      err = stage_source<T>(op, other, res, t0 + n * dt, dt, i, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_step: point-source launch");
       std::swap(cur, other);
     }
   }
-  if (cur != q) {
-    cudaError_t err = cudaMemcpyAsync(q, cur, 3 * op->fstride * sizeof(T),
-                                      cudaMemcpyDeviceToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "dg_step: copy-back");
-  }
+  *result = cur;
+  return DG_OK;
+}
+
+// The same with the result in q.
+template <typename T>
+dg_status run_steps(const dg_op* op, T* q, T* tmp, T* res, double t0, double dt, int32_t nsteps,
+                    cudaStream_t s, const char* where) {
+  T* cur = nullptr;
+  const dg_status st = run_stages<T>(op, q, tmp, res, t0, dt, nsteps, s, &cur, where);
+  if (st != DG_OK || cur == q) return st;
+  cudaError_t err = cudaMemcpyAsync(q, cur, 3 * op->fstride * sizeof(T), cudaMemcpyDeviceToDevice,
+                                    s);
+  if (err != cudaSuccess) return cuda_fail(err, where);
   return DG_OK;
 }
 
@@ -938,30 +927,17 @@ extern "C" dg_status dg_rhs(const dg_op* op, const void* d_q, void* d_rhs, doubl
     dgw::StageArgs<float> a = base_args<float>(op);
     a.qin = static_cast<const float*>(d_q);
     a.rhs = static_cast<float*>(d_rhs);
+    set_source<float>(op, a, t, 1.0);
     err = launch_order<float>(op, a, dgw::kModeRhs, s);
   } else {
     dgw::StageArgs<double> a = base_args<double>(op);
     a.qin = static_cast<const double*>(d_q);
     a.rhs = static_cast<double*>(d_rhs);
+    set_source<double>(op, a, t, 1.0);
     err = launch_order<double>(op, a, dgw::kModeRhs, s);
   }
   if (err != cudaSuccess) return cuda_fail(err, "dg_rhs: kernel launch");
   op->launches.fetch_add(1, std::memory_order_relaxed);
-  if (op->has_src) {
-    const int64_t off = 2 * op->fstride + op->src_k * op->Np;
-    const double pif = M_PI * op->src.f;
-    if (op->precision == DG_FP32)
-      point_source_kernel<float><<<1, 64, 0, s>>>(
-          static_cast<float*>(d_rhs) + off, nullptr, static_cast<const float*>(op->d_src_w),
-          op->Np, t, pif, op->src.t0, op->src.amplitude, 0.0, 0.0, 1);
-    else
-      point_source_kernel<double><<<1, 64, 0, s>>>(
-          static_cast<double*>(d_rhs) + off, nullptr, static_cast<const double*>(op->d_src_w),
-          op->Np, t, pif, op->src.t0, op->src.amplitude, 0.0, 0.0, 1);
-    err = cudaGetLastError();
-    if (err != cudaSuccess) return cuda_fail(err, "dg_rhs: point-source launch");
-    op->launches.fetch_add(1, std::memory_order_relaxed);
-  }
   return DG_OK;
 }
 
@@ -981,10 +957,10 @@ extern "C" dg_status dg_step(const dg_op* op, void* d_q, void* d_res, double t0,
     return fail(DG_ERR_ARG, "dg_step: buffer overlaps the operator's internal buffer");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (op->precision == DG_FP32)
-    return run_steps<float>(op, static_cast<float*>(d_q), static_cast<float*>(d_res), t0, dt,
-                            nsteps, s);
-  return run_steps<double>(op, static_cast<double*>(d_q), static_cast<double*>(d_res), t0, dt,
-                           nsteps, s);
+    return run_steps<float>(op, static_cast<float*>(d_q), static_cast<float*>(op->d_qtmp),
+                            static_cast<float*>(d_res), t0, dt, nsteps, s, "dg_step");
+  return run_steps<double>(op, static_cast<double*>(d_q), static_cast<double*>(op->d_qtmp),
+                           static_cast<double*>(d_res), t0, dt, nsteps, s, "dg_step");
 }
 
 extern "C" dg_status dg_solve(const dg_op* op, void* d_q, void* d_res, double T, double dt,
@@ -1030,35 +1006,6 @@ extern "C" dg_status dg_step_host(const dg_op* op, void* h_q, void* d_q, void* d
 }
 
 namespace {
-
-// nsteps LSRK steps ping-ponging between q and tmp (no copy back); returns
-// the buffer that holds the result
-template <typename T>
-dg_status run_stages(const dg_op* op, T* q, T* tmp, T* res, double t0, double dt,
-                     int32_t nsteps, cudaStream_t s, T** result) {
-  dgw::StageArgs<T> a = base_args<T>(op);
-  a.res = res;
-  a.dt = static_cast<T>(dt);
-  T* cur = q;
-  T* other = tmp;
-  for (int32_t n = 0; n < nsteps; ++n) {
-    for (int i = 0; i < 5; ++i) {
-      a.qin = cur;
-      a.qout = other;
-      a.a = static_cast<T>(op->lsrk_a[i]);
-      a.b = static_cast<T>(op->lsrk_b[i]);
-      const int mode = (i == 0) ? dgw::kModeFirstStage : dgw::kModeStage;
-      cudaError_t err = launch_order<T>(op, a, mode, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_step_host_jobs: kernel launch");
-      op->launches.fetch_add(1, std::memory_order_relaxed);
-      err = stage_source<T>(op, other, res, t0 + n * dt, dt, i, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_step_host_jobs: point-source launch");
-      std::swap(cur, other);
-    }
-  }
-  *result = cur;
-  return DG_OK;
-}
 
 // Pipeline of dg_step_host_jobs: slot j % kJobSlots of the work buffer holds
 // job j's fields (q, tmp); the residual is shared (the first stage of a step
@@ -1139,7 +1086,7 @@ dg_status run_jobs(const dg_op* op, int32_t njobs, void* const* h_q, T* work, do
     if (err == cudaSuccess) err = cudaStreamWaitEvent(s, pipe.in_done[slot], 0);
     if (err != cudaSuccess) return cuda_fail(err, where);
     T* out = nullptr;
-    dg_status st = run_stages<T>(op, q, tmp, res, t0, dt, nsteps, s, &out);
+    dg_status st = run_stages<T>(op, q, tmp, res, t0, dt, nsteps, s, &out, where);
     if (st) return st;
     err = cudaEventRecord(pipe.comp_done[slot], s);
     if (err == cudaSuccess) err = cudaStreamWaitEvent(pipe.d2h, pipe.comp_done[slot], 0);
@@ -1330,38 +1277,6 @@ dg_status static_scratch(int device, void** out) {
   return DG_OK;
 }
 
-// Same launch sequence as run_steps, with `tmp` as the ping-pong buffer.
-template <typename T>
-dg_status run_steps_static(const dg_op* op, T* q, T* res, double t0, double dt, int32_t nsteps,
-                           T* tmp, cudaStream_t s) {
-  dgw::StageArgs<T> a = base_args<T>(op);
-  a.res = res;
-  a.dt = static_cast<T>(dt);
-  T* cur = q;
-  T* other = tmp;
-  for (int32_t n = 0; n < nsteps; ++n) {
-    for (int i = 0; i < 5; ++i) {
-      a.qin = cur;
-      a.qout = other;
-      a.a = static_cast<T>(op->lsrk_a[i]);
-      a.b = static_cast<T>(op->lsrk_b[i]);
-      const int mode = (i == 0) ? dgw::kModeFirstStage : dgw::kModeStage;
-      cudaError_t err = launch_order<T>(op, a, mode, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_step_static: kernel launch");
-      op->launches.fetch_add(1, std::memory_order_relaxed);
-      err = stage_source<T>(op, other, res, t0 + n * dt, dt, i, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_step_static: point-source launch");
-      std::swap(cur, other);
-    }
-  }
-  if (cur != q) {
-    cudaError_t err = cudaMemcpyAsync(q, cur, 3 * op->fstride * sizeof(T),
-                                      cudaMemcpyDeviceToDevice, s);
-    if (err != cudaSuccess) return cuda_fail(err, "dg_step_static: copy-back");
-  }
-  return DG_OK;
-}
-
 }  // namespace
 
 extern "C" dg_status dg_step_static(const dg_op* op, void* d_q, void* d_res, double t0,
@@ -1402,10 +1317,10 @@ extern "C" dg_status dg_step_static(const dg_op* op, void* d_q, void* d_res, dou
     }
   }
   if (op->precision == DG_FP32)
-    return run_steps_static<float>(op, static_cast<float*>(d_q), static_cast<float*>(d_res), t0,
-                                   dt, nsteps, static_cast<float*>(scratch), s);
-  return run_steps_static<double>(op, static_cast<double*>(d_q), static_cast<double*>(d_res), t0,
-                                  dt, nsteps, static_cast<double*>(scratch), s);
+    return run_steps<float>(op, static_cast<float*>(d_q), static_cast<float*>(scratch),
+                            static_cast<float*>(d_res), t0, dt, nsteps, s, "dg_step_static");
+  return run_steps<double>(op, static_cast<double*>(d_q), static_cast<double*>(scratch),
+                           static_cast<double*>(d_res), t0, dt, nsteps, s, "dg_step_static");
 }
 
 namespace dgw {

@@ -115,6 +115,33 @@ __device__ __forceinline__ void load_vec(T (&dst)[W], const T* src) {
 
 __host__ __device__ constexpr uint32_t round16(uint32_t x) { return (x + 15u) & ~15u; }
 
+// sum that no product is fused into
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
+// Launch of a stage kernel that may begin its prologue (barriers, tensor
+// memory, reference tables: nothing another kernel writes) before the launch
+// in front of it in the stream has ended; the kernel calls chain_wait before
+// it touches fields.  A step is a chain of such launches.  Back to back on
+// GB300 an ordinary launch of a few microseconds starts on a 2.05 us grid
+// (4.1 us per launch for 0.5 to 2 us of work, 6.15 for 3.9), a chained one
+// about 0.7 us after its predecessor's last block.
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem,
+                           cudaStream_t stream, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // ------------------------------------------------------------ kernel
 // Offsets inside one field are 32-bit (the host guarantees field_stride <
 // 2^31); each field has its own 64-bit base pointer.  MEDIA: geometry
@@ -183,11 +210,6 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
     tma_load_1d(st + 6 * L::QB + L::GB, p.conn + static_cast<int64_t>(k0) * 3, cb, &bars[s]);
   };
 
-  int issued = 0;  // (thread 0) iterations whose loads were issued
-  if (t == 0) {
-    for (; issued < niter && issued < kStages; ++issued) issue(issued);
-  }
-
   // this thread's rows of Dr, Ds and LIFT, kept in registers
   const T lam2 = __ldg(p.lam + i), lam3 = __ldg(p.lam + Np + i);
   T dr[Np], ds[Np], lf[Nafp];
@@ -211,6 +233,13 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
     task_jj[u] = task_j[u] - task_f[u] * Nfp;
   }
 
+  chain_wait();
+  chain_trigger();
+  int issued = 0;  // (thread 0) iterations whose loads were issued
+  if (t == 0) {
+    for (; issued < niter && issued < kStages; ++issued) issue(issued);
+  }
+
   // neighbour traces of this thread's flux tasks, one block ahead
   T trc[TPT][3];
   auto gather = [&](int it) {
@@ -232,9 +261,9 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
 #endif
         if (code >= 0) {
           const int gP = (code >> 3) * Np + nbr[(code & 7) * Nfp + task_jj[u]];
-          trc[u][0] = __ldg(qin[0] + gP);
-          trc[u][1] = __ldg(qin[1] + gP);
-          trc[u][2] = __ldg(qin[2] + gP);
+          trc[u][0] = qin[0][gP];  // written by the launch before: not the read-only path
+          trc[u][1] = qin[1][gP];
+          trc[u][2] = qin[2][gP];
         }
       }
     }
@@ -443,6 +472,22 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
         p.qout[p.fstride + g] = hy + p.b * n1;
         p.qout[2 * p.fstride + g] = ez + p.b * n2;
       }
+      // the operator's point source, on what this thread has just written
+      // (kept out of the update itself, where it held registers: FP64 at
+      // N = 5 ran 1.5 % slower)
+      if (k0 + e == p.psrc_k) {
+        const T w = p.psrc_w[i];
+        if (MODE == kModeRhs) {
+          T* y = p.rhs + 2 * p.fstride + g;
+          *y = fma(p.psrc_amp, w, *y);
+        } else {
+          T* y = p.qout + 2 * p.fstride + g;
+          T* r = p.res + 2 * p.fstride + g;
+          const T v = p.psrc_amp * w;
+          *r = add_rn(*r, v);
+          *y = fma(p.b, v, *y);
+        }
+      }
     }
   }
 
@@ -479,9 +524,8 @@ cudaError_t launch_stage_mode(const StageArgs<T>& args, int num_sms, cudaStream_
   int64_t grid = static_cast<int64_t>(blocks_per_sm.load()) * num_sms;
   if (grid > nblk) grid = nblk;
   if (grid < 1) grid = 1;
-  dg_stage_kernel<T, N, MODE, MEDIA>
-      <<<static_cast<unsigned>(grid), L::THREADS, L::SMEM_BYTES, stream>>>(args);
-  return cudaGetLastError();
+  return launch_chained(dg_stage_kernel<T, N, MODE, MEDIA>, static_cast<unsigned>(grid),
+                        L::THREADS, L::SMEM_BYTES, stream, args);
 }
 
 template <typename T, int N, bool MEDIA>

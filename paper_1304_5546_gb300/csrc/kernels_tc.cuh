@@ -535,10 +535,52 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  auto fetch_tiles = [&]() {  // the operator tiles, which no kernel writes
+    mbar_expect_tx(op_bar, L::NS * L::OB);
+    tma_load_1d(smem + L::OFF_OP, p.tc_op, L::NS * L::OB, op_bar);
+  };
+  // in a chain the tiles land while the launch before still runs; a batched
+  // launch is not chained, and its memory warp fetches them as it starts
+  // (here they measured 1.4 % slower there)
+  if (!TABLE && warp == L::IO_WARP && lane == 0 && !p.stall_gate) fetch_tiles();
+  if constexpr (!TABLE) {
+    chain_wait();
+    chain_trigger();
+  }
 
   auto fail = [&]() {
     *abort_flag = 1;
     atomicOr(p.status, kStatusTimeout);
+  };
+
+  // The operator's own point source, added by the memory warp (threads l0,
+  // l0 + step, ... of it) to a block's outputs before they leave: in the
+  // stage buffer, or in global memory for the ragged last block.  In the
+  // epilogue, whose registers are all taken, the same few lines cost every
+  // launch 6 % (N = 5, K = 1.0M: 1179 against 1112 us a step).
+  auto add_source = [&](int k0, int nv, float* sq, int l0, int step) {
+    if constexpr (!TABLE) {
+      const int e = p.psrc_k - k0;
+      if (p.psrc_k < 0 || e < 0 || e >= nv) return;
+      float* y = sq + 2 * E * Np + e * Np;  // Ez values (or right-hand side)
+      float* r = y + 3 * E * Np;
+      if (nv != E) {
+        const int64_t g = 2 * fs + static_cast<int64_t>(p.psrc_k) * Np;
+        y = (MODE == kModeRhs ? p.rhs : p.qout) + g;
+        r = p.res + g;
+      }
+      for (int n = l0; n < Np; n += step) {
+        const float w = __ldg(p.psrc_w + n);
+        if (MODE == kModeRhs) {
+          y[n] = __fmaf_rn(p.psrc_amp, w, y[n]);
+        } else {
+          const float v = __fmul_rn(p.psrc_amp, w);
+          r[n] = __fadd_rn(r[n], v);
+          y[n] = __fmaf_rn(p.b, v, y[n]);
+        }
+      }
+      fence_proxy_async();
+    }
   };
 
   if (warp == L::IO_WARP) {
@@ -588,10 +630,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
       if (ok) {
-        if (lane == 0) {
-          mbar_expect_tx(op_bar, L::NS * L::OB);
-          tma_load_1d(smem + L::OFF_OP, p.tc_op, L::NS * L::OB, op_bar);
-        }
+        if ((TABLE || p.stall_gate) && lane == 0) fetch_tiles();
         for (; issued < niter && issued < S; ++issued) issue(issued);
       }
       for (int jj = 0; ok && jj < niter; ++jj) {
@@ -602,6 +641,10 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
         if (!ok) break;
         int k0, nv;
         block_at(jj, k0, nv);
+        if constexpr (!TABLE) {
+          add_source(k0, nv, reinterpret_cast<float*>(stages + s * L::STAGE_BYTES), lane, 32);
+          __syncwarp();
+        }
         if (nv == E && lane < 6) {
           const float* sq = reinterpret_cast<const float*>(stages + s * L::STAGE_BYTES);
           if (MODE == kModeRhs) {
@@ -669,8 +712,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           }
         }
         if (ok) {
-          mbar_expect_tx(op_bar, L::NS * L::OB);
-          tma_load_1d(smem + L::OFF_OP, p.tc_op, L::NS * L::OB, op_bar);
+          if (TABLE || p.stall_gate) fetch_tiles();
           for (; issued < niter && issued < S; ++issued) issue(issued);
         }
         // outputs of block jj leave by bulk stores, one bulk group per block
@@ -683,6 +725,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           if (!ok) break;
           int k0, nv;
           block_at(jj, k0, nv);
+          if constexpr (!TABLE)
+            add_source(k0, nv, reinterpret_cast<float*>(stages + s * L::STAGE_BYTES), 0, 1);
           if (nv == E) {
             const float* sq = reinterpret_cast<const float*>(stages + s * L::STAGE_BYTES);
             if (MODE == kModeRhs) {
@@ -822,9 +866,11 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           if (code >= 0 && !(PAIRS && static_cast<unsigned>((code >> 3) - k0) <
                                            static_cast<unsigned>(nv))) {
             const int gP = (code >> 3) * Np + nbr[(code & 7) * Nfp + task_jj[u]];
-            trc[u][0] = __ldg(qin[0] + gP);
-            trc[u][1] = __ldg(qin[1] + gP);
-            trc[u][2] = __ldg(qin[2] + gP);
+            // a chained launch starts while the one before still writes these:
+            // not the read-only path
+            trc[u][0] = TABLE ? __ldg(qin[0] + gP) : qin[0][gP];
+            trc[u][1] = TABLE ? __ldg(qin[1] + gP) : qin[1][gP];
+            trc[u][2] = TABLE ? __ldg(qin[2] + gP) : qin[2][gP];
           }
         }
       }
@@ -1245,9 +1291,8 @@ cudaError_t launch_stage_tc_mode(const StageArgs<float>& args, int num_sms, cuda
   int64_t grid = num_sms;  // one CTA per SM (shared memory and TMEM sized for it)
   if (grid > nblk) grid = nblk;
   if (grid < 1) grid = 1;
-  dg_stage_tc_kernel<N, MODE, PREC, MEDIA, PAIRS, ALT>
-      <<<static_cast<unsigned>(grid), L::THREADS, L::SMEM_BYTES, stream>>>(args);
-  return cudaGetLastError();
+  return launch_chained(dg_stage_tc_kernel<N, MODE, PREC, MEDIA, PAIRS, ALT>,
+                        static_cast<unsigned>(grid), L::THREADS, L::SMEM_BYTES, stream, args);
 }
 
 template <int N, int PREC, bool MEDIA, bool PAIRS, bool ALT = false>

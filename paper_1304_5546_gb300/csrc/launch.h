@@ -127,6 +127,13 @@ struct StageArgs {
   const int* src_step = nullptr;
   const int* step_ctr = nullptr;
   double c_stage = 0.0;
+  // point source of a single operator (dg_operator_set_source): element
+  // psrc_k (-1: none) gains psrc_amp * psrc_w[n] in its Ez residual, and b
+  // times that in its Ez values (psrc_amp = dt s(t)); kModeRhs: in its Ez
+  // right-hand side (psrc_amp = s(t))
+  int psrc_k = -1;
+  T psrc_amp = 0;
+  const T* psrc_w = nullptr;
   // tensor-core path only: [Dr | Ds | LIFT | 1] as the operator tiles of the
   // launch's product variant (tc_nsplit tiles of tc_nn(N) x tc_kpp(N, prec)
   // elements, TF32 or BF16, in the core-matrix layout of tc_canon /

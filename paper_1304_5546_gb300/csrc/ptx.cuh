@@ -65,6 +65,23 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
+// Programmatic dependent launch (the stage launches of a chain, see
+// launch_chained): wait returns once every kernel this launch depends on has
+// completed and its writes are visible; until then nothing that such a
+// kernel writes may be read, and nothing that it reads may be written.
+// trigger lets the next launch of the chain start its own prologue (without
+// it that launch starts as this one's last block ends).  It is called after
+// wait only, so at most two launches of a chain are resident at a time, and
+// by the time a launch starts, the one before its predecessor has ended: no
+// line that the L1 of an SM holds of that launch's input (the buffer its
+// predecessor writes) can be filled after the launch began.
+__device__ __forceinline__ void chain_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void chain_trigger() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // Wait for phase `parity` of `bar`; false if it has not completed in limit_ns.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity,
                                                   unsigned long long limit_ns) {
