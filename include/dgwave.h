@@ -309,7 +309,8 @@ dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems);
 
 /* dg_operator_kernel: the kernel the operator's hot-path calls run
  * (DG_KERNEL_*) and its elements per block (the element-thread kernel: 32,
- * one per lane of a warp).  Errors: DG_ERR_ARG (NULL).                    */
+ * one per lane of a warp; the FP64 kernel: the most a block holds, smaller
+ * meshes take smaller blocks).  Errors: DG_ERR_ARG (NULL).                */
 #define DG_KERNEL_TENSOR_CORES 0
 #define DG_KERNEL_CUDA_CORES 1
 #define DG_KERNEL_ELEMENT_THREADS 2

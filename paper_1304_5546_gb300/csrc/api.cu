@@ -174,6 +174,42 @@ namespace {
 
 using dgw::tc_operator_tiles;
 
+// Dr, Ds and LIFT in fixed point for the FP64 kernel (f64_table_pairs,
+// launch.h): v = (hi 2^28 + lo) 2^scale, at most 2^55 in size, with a scale
+// per node for its rows of Dr and Ds and one for its row of LIFT.
+std::vector<unsigned char> f64_operator_table(const dgw::RefElement& R) {
+  const int N = R.N, Np = R.Np, Nafp = R.Nafp;
+  std::vector<int> sd(Np), sl(Np);
+  for (int n = 0; n < Np; ++n) {
+    double d = 0.0, l = 0.0;
+    for (int m = 0; m < Np; ++m)
+      d = std::max({d, std::fabs(R.Dr[n * Np + m]), std::fabs(R.Ds[n * Np + m])});
+    for (int j = 0; j < Nafp; ++j) l = std::max(l, std::fabs(R.LIFT[n * Nafp + j]));
+    sd[n] = std::ilogb(d) + 1 - 55;
+    sl[n] = std::ilogb(l) + 1 - 55;
+  }
+  std::vector<int32_t> out;
+  auto put = [&](double v, int scale) {
+    const int64_t n = std::llround(std::ldexp(v, -scale));
+    const int64_t lo = ((n + (1 << 27)) & ((1 << 28) - 1)) - (1 << 27);
+    out.push_back(static_cast<int32_t>((n - lo) >> 28));
+    out.push_back(static_cast<int32_t>(lo));
+  };
+  for (const std::vector<double>* D : {&R.Dr, &R.Ds})
+    for (int c = 0; c < Np - 3; ++c)
+      for (int n = 0; n < Np; ++n) put((*D)[n * Np + (c < N - 1 ? c + 1 : c + 2)], sd[n]);
+  for (int j = 0; j < Nafp; ++j)
+    for (int n = 0; n < Np; ++n) put(R.LIFT[n * Nafp + j], sl[n]);
+  out.resize(2 * static_cast<size_t>(dgw::f64_table_pairs(N)), 0);
+  for (int n = 0; n < Np; ++n) {
+    out.push_back(sd[n]);
+    out.push_back(sl[n]);
+  }
+  std::vector<unsigned char> bytes(out.size() * 4);
+  std::memcpy(bytes.data(), out.data(), bytes.size());
+  return bytes;
+}
+
 template <typename T>
 dg_status upload(dg_op* op, const std::vector<double>& rec_in,
                  const std::vector<int32_t>& conn_in) {
@@ -228,8 +264,9 @@ dg_status upload(dg_op* op, const std::vector<double>& rec_in,
   if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMemset");
   err = dgw::dev_malloc(&op->d_flag, sizeof(int));
   if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMalloc(flag)");
-  if (op->use_tc) {
-    const std::vector<unsigned char> tiles = tc_operator_tiles(op->ref, op->tc_prec);
+  if (op->use_tc || sizeof(T) == 8) {
+    const std::vector<unsigned char> tiles =
+        sizeof(T) == 8 ? f64_operator_table(op->ref) : tc_operator_tiles(op->ref, op->tc_prec);
     err = dgw::dev_malloc(&op->d_tcop, tiles.size());
     if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMalloc(operator tiles)");
     err = cudaMemcpy(op->d_tcop, tiles.data(), tiles.size(), cudaMemcpyHostToDevice);
@@ -299,21 +336,18 @@ cudaError_t launch_order_ept_media(const dg_op* op, const dgw::StageArgs<float>&
   }
 }
 
-template <typename T>
-cudaError_t launch_order_media(const dg_op* op, const dgw::StageArgs<T>& a, int mode,
+cudaError_t launch_order_media(const dg_op* op, const dgw::StageArgs<float>& a, int mode,
                                cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {
-    if (op->use_ept) return launch_order_ept_media(op, a, mode, s);
-    if (op->use_tc) return launch_order_tc_media(op, a, mode, s);
-  }
+  if (op->use_ept) return launch_order_ept_media(op, a, mode, s);
+  if (op->use_tc) return launch_order_tc_media(op, a, mode, s);
   switch (op->N) {
-    case 1: return dgw::launch_stage_media<T, 1>(a, mode, op->num_sms, s);
-    case 2: return dgw::launch_stage_media<T, 2>(a, mode, op->num_sms, s);
-    case 3: return dgw::launch_stage_media<T, 3>(a, mode, op->num_sms, s);
-    case 4: return dgw::launch_stage_media<T, 4>(a, mode, op->num_sms, s);
-    case 5: return dgw::launch_stage_media<T, 5>(a, mode, op->num_sms, s);
-    case 6: return dgw::launch_stage_media<T, 6>(a, mode, op->num_sms, s);
-    case 7: return dgw::launch_stage_media<T, 7>(a, mode, op->num_sms, s);
+    case 1: return dgw::launch_stage_media<1>(a, mode, op->num_sms, s);
+    case 2: return dgw::launch_stage_media<2>(a, mode, op->num_sms, s);
+    case 3: return dgw::launch_stage_media<3>(a, mode, op->num_sms, s);
+    case 4: return dgw::launch_stage_media<4>(a, mode, op->num_sms, s);
+    case 5: return dgw::launch_stage_media<5>(a, mode, op->num_sms, s);
+    case 6: return dgw::launch_stage_media<6>(a, mode, op->num_sms, s);
+    case 7: return dgw::launch_stage_media<7>(a, mode, op->num_sms, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -335,20 +369,31 @@ cudaError_t launch_order_ept(const dg_op* op, const dgw::StageArgs<float>& a, in
 
 template <typename T>
 cudaError_t launch_order(const dg_op* op, const dgw::StageArgs<T>& a, int mode, cudaStream_t s) {
-  if (op->media()) return launch_order_media<T>(op, a, mode, s);
-  if constexpr (sizeof(T) == 4) {
+  if constexpr (sizeof(T) == 8) {
+    switch (op->N) {
+      case 1: return dgw::launch_stage_f64<1>(a, op->media(), mode, op->num_sms, s);
+      case 2: return dgw::launch_stage_f64<2>(a, op->media(), mode, op->num_sms, s);
+      case 3: return dgw::launch_stage_f64<3>(a, op->media(), mode, op->num_sms, s);
+      case 4: return dgw::launch_stage_f64<4>(a, op->media(), mode, op->num_sms, s);
+      case 5: return dgw::launch_stage_f64<5>(a, op->media(), mode, op->num_sms, s);
+      case 6: return dgw::launch_stage_f64<6>(a, op->media(), mode, op->num_sms, s);
+      case 7: return dgw::launch_stage_f64<7>(a, op->media(), mode, op->num_sms, s);
+      default: return cudaErrorInvalidValue;
+    }
+  } else {
+    if (op->media()) return launch_order_media(op, a, mode, s);
     if (op->use_ept) return launch_order_ept(op, a, mode, s);
     if (op->use_tc) return launch_order_tc(op, a, mode, s);
-  }
-  switch (op->N) {
-    case 1: return dgw::launch_stage<T, 1>(a, mode, op->num_sms, s);
-    case 2: return dgw::launch_stage<T, 2>(a, mode, op->num_sms, s);
-    case 3: return dgw::launch_stage<T, 3>(a, mode, op->num_sms, s);
-    case 4: return dgw::launch_stage<T, 4>(a, mode, op->num_sms, s);
-    case 5: return dgw::launch_stage<T, 5>(a, mode, op->num_sms, s);
-    case 6: return dgw::launch_stage<T, 6>(a, mode, op->num_sms, s);
-    case 7: return dgw::launch_stage<T, 7>(a, mode, op->num_sms, s);
-    default: return cudaErrorInvalidValue;
+    switch (op->N) {
+      case 1: return dgw::launch_stage<1>(a, mode, op->num_sms, s);
+      case 2: return dgw::launch_stage<2>(a, mode, op->num_sms, s);
+      case 3: return dgw::launch_stage<3>(a, mode, op->num_sms, s);
+      case 4: return dgw::launch_stage<4>(a, mode, op->num_sms, s);
+      case 5: return dgw::launch_stage<5>(a, mode, op->num_sms, s);
+      case 6: return dgw::launch_stage<6>(a, mode, op->num_sms, s);
+      case 7: return dgw::launch_stage<7>(a, mode, op->num_sms, s);
+      default: return cudaErrorInvalidValue;
+    }
   }
 }
 
@@ -392,7 +437,8 @@ int block_elems(const dg_op* op, int alt) {
   if (op->precision == DG_FP32 && op->use_ept) return 32;
   if (op->precision == DG_FP32 && op->use_tc)
     return 40 * dgw::tc_tiles(op->N, op->tc_prec, alt != 0 && op->tc_prec == dgw::kTcTf32x3);
-  return dgw::simt_block_elems(op->N, op->precision == DG_FP64);
+  if (op->precision == DG_FP64) return dgw::f64_max_elems(op->N);
+  return dgw::simt_block_elems(op->N);
 }
 
 dg_status check_device_op(const dg_op* op, const char* where) {

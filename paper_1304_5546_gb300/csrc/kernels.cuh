@@ -1,4 +1,5 @@
-// Fused nodal-DG stage kernel for the 2D TM Maxwell system.
+// Fused nodal-DG stage kernel for the 2D TM Maxwell system: FP32, one thread
+// per (element, node), on the CUDA cores.
 //
 // One launch evaluates the right-hand side of Eq. dg-strong-explicit for
 // every element -- the volume derivative (Dr/Ds and the chain rule of
@@ -51,45 +52,26 @@ struct Order {
   static constexpr int Nafp = 3 * (N + 1);
 };
 
-// Elements per block: simt_block_elems (launch.h, with the reasons).
-template <typename T, int N>
-constexpr int elems_per_block() {
-  return simt_block_elems(N, sizeof(T) == 8);
-}
-
 constexpr int kStages = 3;
-
-template <typename T>
-struct Vec16;
-template <>
-struct Vec16<float> {
-  using type = float4;
-  static constexpr int width = 4;
-};
-template <>
-struct Vec16<double> {
-  using type = double2;
-  static constexpr int width = 2;
-};
 
 constexpr int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-template <typename T, int N, bool MEDIA = false>
+template <int N, bool MEDIA = false>
 struct Layout {
   static constexpr int GEO = MEDIA ? kGeoMedia : kGeo;  // geometry record length
   static constexpr int Np = Order<N>::Np;
   static constexpr int Nfp = Order<N>::Nfp;
   static constexpr int Nafp = Order<N>::Nafp;
-  static constexpr int E = elems_per_block<T, N>();
-  static constexpr int VW = Vec16<T>::width;
+  static constexpr int E = simt_block_elems(N);
+  static constexpr int VW = 4;
   static constexpr int NPAD = round_up(Np, VW);
   static constexpr int FPAD = round_up(Nafp, VW);
   static constexpr int THREADS = E * Np;
   static constexpr int TASKS = E * Nafp;                       // flux tasks per block
   static constexpr int TPT = (TASKS + THREADS - 1) / THREADS;  // per thread
   // stage buffer: q[3][E Np], res[3][E Np], geo[E][kGeo], conn[E][3]
-  static constexpr int QB = E * Np * static_cast<int>(sizeof(T));
-  static constexpr int GB = E * GEO * static_cast<int>(sizeof(T));
+  static constexpr int QB = E * Np * 4;
+  static constexpr int GB = E * GEO * 4;
   static constexpr int CB = E * 3 * 4;
   static constexpr int STAGE_BYTES = round_up(6 * QB + GB + CB, 128);
   // double-buffered work arrays: centred volume operands and lifted fluxes
@@ -98,7 +80,7 @@ struct Layout {
   static constexpr int HEADER = 512;  // mbarriers + neighbour face-node table
   static_assert(64 + 6 * Nfp * 4 <= HEADER, "header");
   static constexpr size_t SMEM_BYTES =
-      HEADER + kStages * STAGE_BYTES + 2 * sizeof(T) * (W_ELEMS + F_ELEMS);
+      HEADER + kStages * STAGE_BYTES + 2 * sizeof(float) * (W_ELEMS + F_ELEMS);
   static_assert(QB % 16 == 0 && GB % 16 == 0 && CB % 16 == 0, "16-byte TMA chunks");
 };
 
@@ -107,17 +89,11 @@ __host__ __device__ constexpr int face_node_dev(int N, int f, int j) {
                 : (f == 1 ? j * (N + 1) - j * (j - 1) / 2 + (N - j) : j * (N + 1) - j * (j - 1) / 2);
 }
 
-template <typename T, int W>
-__device__ __forceinline__ void load_vec(T (&dst)[W], const T* src) {
-  using V = typename Vec16<T>::type;
-  *reinterpret_cast<V*>(dst) = *reinterpret_cast<const V*>(src);
+__device__ __forceinline__ void load_vec(float (&dst)[4], const float* src) {
+  *reinterpret_cast<float4*>(dst) = *reinterpret_cast<const float4*>(src);
 }
 
 __host__ __device__ constexpr uint32_t round16(uint32_t x) { return (x + 15u) & ~15u; }
-
-// sum that no product is fused into
-__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
-__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
 
 // Launch of a stage kernel that may begin its prologue (barriers, tensor
 // memory, reference tables: nothing another kernel writes) before the launch
@@ -148,10 +124,10 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads
 // records of kGeoMedia values (per-element permittivity, see launch.h): the
 // flux of the exact interface Riemann solution and per-row scales of the
 // right-hand side.
-template <typename T, int N, int MODE, bool MEDIA>
-__global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
-    dg_stage_kernel(const StageArgs<T> p) {
-  using L = Layout<T, N, MEDIA>;
+template <int N, int MODE, bool MEDIA>
+__global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
+    dg_stage_kernel(const StageArgs<float> p) {
+  using L = Layout<N, MEDIA>;
   constexpr int GEO = L::GEO;
   constexpr int Np = L::Np, Nfp = L::Nfp, Nafp = L::Nafp;
   constexpr int E = L::E, NPAD = L::NPAD, FPAD = L::FPAD, VW = L::VW;
@@ -162,8 +138,8 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem);
   int* nbr = reinterpret_cast<int*>(smem + 64);  // [6][Nfp] neighbour face-node table
   unsigned char* stages = smem + L::HEADER;
-  T* Wbuf = reinterpret_cast<T*>(stages + kStages * L::STAGE_BYTES);  // [2][3][E][NPAD]
-  T* Fbuf = Wbuf + 2 * L::W_ELEMS;                                    // [2][3][E][FPAD]
+  float* Wbuf = reinterpret_cast<float*>(stages + kStages * L::STAGE_BYTES);  // [2][3][E][NPAD]
+  float* Fbuf = Wbuf + 2 * L::W_ELEMS;                                    // [2][3][E][FPAD]
 
   const int t = threadIdx.x;
   const int e = t / Np;
@@ -174,7 +150,7 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
   const int G = gridDim.x;
   const int first = blockIdx.x;
   const int niter = first < nblk ? (nblk - 1 - first) / G + 1 : 0;
-  const T* qin[3] = {p.qin, p.qin + p.fstride, p.qin + 2 * p.fstride};
+  const float* qin[3] = {p.qin, p.qin + p.fstride, p.qin + 2 * p.fstride};
 
   if (t == 0) {
     for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
@@ -193,8 +169,8 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
     const int s = it % kStages;
     const int k0 = (first + it * G) * E;
     const int n = (K - k0) < E ? (K - k0) : E;
-    const uint32_t qb = round16(static_cast<uint32_t>(n * Np * sizeof(T)));
-    const uint32_t gb = round16(static_cast<uint32_t>(n * GEO * sizeof(T)));
+    const uint32_t qb = round16(static_cast<uint32_t>(n * Np * sizeof(float)));
+    const uint32_t gb = round16(static_cast<uint32_t>(n * GEO * sizeof(float)));
     const uint32_t cb = round16(static_cast<uint32_t>(n * 3 * 4));
     unsigned char* st = stages + s * L::STAGE_BYTES;
     mbar_expect_tx(&bars[s], NQ * qb + gb + cb);
@@ -211,8 +187,8 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
   };
 
   // this thread's rows of Dr, Ds and LIFT, kept in registers
-  const T lam2 = __ldg(p.lam + i), lam3 = __ldg(p.lam + Np + i);
-  T dr[Np], ds[Np], lf[Nafp];
+  const float lam2 = __ldg(p.lam + i), lam3 = __ldg(p.lam + Np + i);
+  float dr[Np], ds[Np], lf[Nafp];
 #pragma unroll
   for (int m = 0; m < Np; ++m) {
     dr[m] = __ldg(p.Dr + i * Np + m);
@@ -241,7 +217,7 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
   }
 
   // neighbour traces of this thread's flux tasks, one block ahead
-  T trc[TPT][3];
+  float trc[TPT][3];
   auto gather = [&](int it) {
     const int s = it % kStages;
     const int32_t* sc =
@@ -249,7 +225,7 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
     const int k0 = (first + it * G) * E;
 #pragma unroll
     for (int u = 0; u < TPT; ++u) {
-      trc[u][0] = trc[u][1] = trc[u][2] = T(0);
+      trc[u][0] = trc[u][1] = trc[u][2] = 0.f;
       const int ee = task_e[u];
       if (ee < E && k0 + ee < K) {
         const int32_t code = sc[ee * 3 + task_f[u]];
@@ -284,17 +260,17 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
     const bool valid = k0 + e < K;
     const int g = k0 * Np + t;  // == k * Np + i
     const unsigned char* st = stages + s * L::STAGE_BYTES;
-    const T* sq = reinterpret_cast<const T*>(st);
-    const T* sg = reinterpret_cast<const T*>(st + 6 * L::QB);
+    const float* sq = reinterpret_cast<const float*>(st);
+    const float* sg = reinterpret_cast<const float*>(st + 6 * L::QB);
     const int32_t* sc = reinterpret_cast<const int32_t*>(st + 6 * L::QB + L::GB);
-    T* Wb = Wbuf + (it & 1) * L::W_ELEMS;
-    T* Fb = Fbuf + (it & 1) * L::F_ELEMS;
+    float* Wb = Wbuf + (it & 1) * L::W_ELEMS;
+    float* Fb = Fbuf + (it & 1) * L::F_ELEMS;
 
     // ---- phase 1: own values, residual, geometry; volume operands minus
     // their linear part
-    T hx = 0, hy = 0, ez = 0, r0 = 0, r1 = 0, r2 = 0, rx = 0, ry = 0, sx = 0, sy = 0;
-    T lin0 = 0, lin1 = 0, lin2 = 0;
-    T sH = 1, sE = 1;  // row scales of the right-hand side (media records)
+    float hx = 0, hy = 0, ez = 0, r0 = 0, r1 = 0, r2 = 0, rx = 0, ry = 0, sx = 0, sy = 0;
+    float lin0 = 0, lin1 = 0, lin2 = 0;
+    float sH = 1, sE = 1;  // row scales of the right-hand side (media records)
     if (ok) {
       hx = sq[t];
       hy = sq[E * Np + t];
@@ -312,20 +288,20 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
         sH = sg[e * GEO + 17];
         sE = sg[e * GEO + 18];
       }
-      const T* qe = sq + e * Np;  // vertex nodes: 0, N, Np - 1
-      const T x1 = qe[0], x2 = qe[N], x3 = qe[Np - 1];
-      const T y1 = qe[E * Np], y2 = qe[E * Np + N], y3 = qe[E * Np + Np - 1];
-      const T z1 = qe[2 * E * Np], z2 = qe[2 * E * Np + N], z3 = qe[2 * E * Np + Np - 1];
-      const T dhx = (hx - x1) - ((x2 - x1) * lam2 + (x3 - x1) * lam3);
-      const T dhy = (hy - y1) - ((y2 - y1) * lam2 + (y3 - y1) * lam3);
+      const float* qe = sq + e * Np;  // vertex nodes: 0, N, Np - 1
+      const float x1 = qe[0], x2 = qe[N], x3 = qe[Np - 1];
+      const float y1 = qe[E * Np], y2 = qe[E * Np + N], y3 = qe[E * Np + Np - 1];
+      const float z1 = qe[2 * E * Np], z2 = qe[2 * E * Np + N], z3 = qe[2 * E * Np + Np - 1];
+      const float dhx = (hx - x1) - ((x2 - x1) * lam2 + (x3 - x1) * lam3);
+      const float dhy = (hy - y1) - ((y2 - y1) * lam2 + (y3 - y1) * lam3);
       Wb[(0 * E + e) * NPAD + i] = (ez - z1) - ((z2 - z1) * lam2 + (z3 - z1) * lam3);
       Wb[(1 * E + e) * NPAD + i] = rx * dhy - ry * dhx;
       Wb[(2 * E + e) * NPAD + i] = sx * dhy - sy * dhx;
       // derivatives of the linear part along r and s
-      const T grz = T(0.5) * (z2 - z1), gsz = T(0.5) * (z3 - z1);
+      const float grz = 0.5f * (z2 - z1), gsz = 0.5f * (z3 - z1);
       lin0 = -(ry * grz + sy * gsz);
       lin1 = rx * grz + sx * gsz;
-      lin2 = T(0.5) * (rx * (y2 - y1) - ry * (x2 - x1) + sx * (y3 - y1) - sy * (x3 - x1));
+      lin2 = 0.5f * (rx * (y2 - y1) - ry * (x2 - x1) + sx * (y3 - y1) - sy * (x3 - x1));
     }
     if (__syncthreads_or(!ok)) break;
 
@@ -336,8 +312,8 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
       if (ee < E && k0 + ee < K) {
         const int f = task_f[u], j = task_j[u];
         const int nM = ee * Np + face_node_dev(N, f, task_jj[u]);
-        const T hxM = sq[nM], hyM = sq[E * Np + nM], ezM = sq[2 * E * Np + nM];
-        T dHx, dHy, dEz;
+        const float hxM = sq[nM], hyM = sq[E * Np + nM], ezM = sq[2 * E * Np + nM];
+        float dHx, dHy, dEz;
         if (sc[ee * 3 + f] < 0) {  // PEC wall: Ez+ = -Ez-, H+ = H-
           dHx = 0;
           dHy = 0;
@@ -349,18 +325,18 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
         }
         if constexpr (MEDIA) {
           // exact interface Riemann solution: fz = cH [Ht] - cE [Ez]
-          const T* gf = sg + ee * GEO + 4 + 4 * f;
-          const T nx = gf[0], ny = gf[1], cH = gf[2], cE = gf[3];
-          const T zM = sg[ee * GEO + 16];
-          const T fz = cH * (ny * dHx - nx * dHy) - cE * dEz;
+          const float* gf = sg + ee * GEO + 4 + 4 * f;
+          const float nx = gf[0], ny = gf[1], cH = gf[2], cE = gf[3];
+          const float zM = sg[ee * GEO + 16];
+          const float fz = cH * (ny * dHx - nx * dHy) - cE * dEz;
           Fb[(0 * E + ee) * FPAD + j] = -zM * ny * fz;
           Fb[(1 * E + ee) * FPAD + j] = zM * nx * fz;
           Fb[(2 * E + ee) * FPAD + j] = fz;
         } else {
           // Eq. max2d-numflux with parameter alpha (1: upwind, 0: central)
-          const T* gf = sg + ee * GEO + 4 + 3 * f;
-          const T nx = gf[0], ny = gf[1], fsc = gf[2], fa = fsc * p.alpha;
-          const T ndotdH = nx * dHx + ny * dHy;
+          const float* gf = sg + ee * GEO + 4 + 3 * f;
+          const float nx = gf[0], ny = gf[1], fsc = gf[2], fa = fsc * p.alpha;
+          const float ndotdH = nx * dHx + ny * dHy;
           Fb[(0 * E + ee) * FPAD + j] = fsc * ny * dEz + fa * (ndotdH * nx - dHx);
           Fb[(1 * E + ee) * FPAD + j] = -fsc * nx * dEz + fa * (ndotdH * ny - dHy);
           Fb[(2 * E + ee) * FPAD + j] = fsc * (ny * dHx - nx * dHy) - fa * dEz;
@@ -383,21 +359,21 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
 
     // ---- phase 3: volume products, lift, stage update (seven independent
     // accumulation chains)
-    T dEzdr = 0, dEzds = 0, cA = 0, cB = 0;
-    T l0 = 0, l1 = 0, l2 = 0;
-    const T* pEz = Wb + (0 * E + e) * NPAD;
-    const T* pA = Wb + (1 * E + e) * NPAD;
-    const T* pB = Wb + (2 * E + e) * NPAD;
-    const T* pF0 = Fb + (0 * E + e) * FPAD;
-    const T* pF1 = Fb + (1 * E + e) * FPAD;
-    const T* pF2 = Fb + (2 * E + e) * FPAD;
+    float dEzdr = 0, dEzds = 0, cA = 0, cB = 0;
+    float l0 = 0, l1 = 0, l2 = 0;
+    const float* pEz = Wb + (0 * E + e) * NPAD;
+    const float* pA = Wb + (1 * E + e) * NPAD;
+    const float* pB = Wb + (2 * E + e) * NPAD;
+    const float* pF0 = Fb + (0 * E + e) * FPAD;
+    const float* pF1 = Fb + (1 * E + e) * FPAD;
+    const float* pF2 = Fb + (2 * E + e) * FPAD;
 #pragma unroll
     for (int m0 = 0; m0 < NPAD; m0 += VW) {
       if (m0 < Np) {
-        T vz[VW], va[VW], vb[VW];
-        load_vec<T, VW>(vz, pEz + m0);
-        load_vec<T, VW>(va, pA + m0);
-        load_vec<T, VW>(vb, pB + m0);
+        float vz[VW], va[VW], vb[VW];
+        load_vec(vz, pEz + m0);
+        load_vec(va, pA + m0);
+        load_vec(vb, pB + m0);
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
           if (m0 + u < Np) {
@@ -409,10 +385,10 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
         }
       }
       if (m0 < Nafp) {
-        T f0[VW], f1[VW], f2[VW];
-        load_vec<T, VW>(f0, pF0 + m0);
-        load_vec<T, VW>(f1, pF1 + m0);
-        load_vec<T, VW>(f2, pF2 + m0);
+        float f0[VW], f1[VW], f2[VW];
+        load_vec(f0, pF0 + m0);
+        load_vec(f1, pF1 + m0);
+        load_vec(f2, pF2 + m0);
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
           if (m0 + u < Nafp) {
@@ -426,10 +402,10 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
     if (FPAD > NPAD) {  // lift columns beyond the volume loop (N = 1, 2)
 #pragma unroll
       for (int m0 = NPAD; m0 < Nafp; m0 += VW) {
-        T f0[VW], f1[VW], f2[VW];
-        load_vec<T, VW>(f0, pF0 + m0);
-        load_vec<T, VW>(f1, pF1 + m0);
-        load_vec<T, VW>(f2, pF2 + m0);
+        float f0[VW], f1[VW], f2[VW];
+        load_vec(f0, pF0 + m0);
+        load_vec(f1, pF1 + m0);
+        load_vec(f2, pF2 + m0);
 #pragma unroll
         for (int u = 0; u < VW; ++u) {
           if (m0 + u < Nafp) {
@@ -440,9 +416,9 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
         }
       }
     }
-    T rhsHx = -(ry * dEzdr + sy * dEzds) + lin0 + l0;
-    T rhsHy = (rx * dEzdr + sx * dEzds) + lin1 + l1;
-    T rhsEz = (cA + cB) + lin2 + l2;
+    float rhsHx = -(ry * dEzdr + sy * dEzds) + lin0 + l0;
+    float rhsHy = (rx * dEzdr + sx * dEzds) + lin1 + l1;
+    float rhsEz = (cA + cB) + lin2 + l2;
     if (MEDIA) {
       rhsHx *= sH;
       rhsHy *= sH;
@@ -455,7 +431,7 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
         p.rhs[p.fstride + g] = rhsHy;
         p.rhs[2 * p.fstride + g] = rhsEz;
       } else {
-        T n0, n1, n2;
+        float n0, n1, n2;
         if (MODE == kModeFirstStage) {
           n0 = p.dt * rhsHx;
           n1 = p.dt * rhsHy;
@@ -476,16 +452,16 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
       // (kept out of the update itself, where it held registers: FP64 at
       // N = 5 ran 1.5 % slower)
       if (k0 + e == p.psrc_k) {
-        const T w = p.psrc_w[i];
+        const float w = p.psrc_w[i];
         if (MODE == kModeRhs) {
-          T* y = p.rhs + 2 * p.fstride + g;
-          *y = fma(p.psrc_amp, w, *y);
+          float* y = p.rhs + 2 * p.fstride + g;
+          *y = fmaf(p.psrc_amp, w, *y);
         } else {
-          T* y = p.qout + 2 * p.fstride + g;
-          T* r = p.res + 2 * p.fstride + g;
-          const T v = p.psrc_amp * w;
-          *r = add_rn(*r, v);
-          *y = fma(p.b, v, *y);
+          float* y = p.qout + 2 * p.fstride + g;
+          float* r = p.res + 2 * p.fstride + g;
+          const float v = p.psrc_amp * w;
+          *r = __fadd_rn(*r, v);
+          *y = fmaf(p.b, v, *y);
         }
       }
     }
@@ -501,20 +477,20 @@ __global__ void __launch_bounds__(Layout<T, N, MEDIA>::THREADS)
   }
 }
 
-template <typename T, int N, int MODE, bool MEDIA>
-cudaError_t launch_stage_mode(const StageArgs<T>& args, int num_sms, cudaStream_t stream) {
-  using L = Layout<T, N, MEDIA>;
-  // per (T, N, MODE, MEDIA): shared-memory attribute and resident CTAs per
+template <int N, int MODE, bool MEDIA>
+cudaError_t launch_stage_mode(const StageArgs<float>& args, int num_sms, cudaStream_t stream) {
+  using L = Layout<N, MEDIA>;
+  // per (N, MODE, MEDIA): shared-memory attribute and resident CTAs per
   // SM, set on the first launch on each device
   static std::atomic<uint64_t> configured{0};
   static std::atomic<int> blocks_per_sm{1};
   cudaError_t err = configure_once_per_device(configured, [] {
-    cudaError_t e = cudaFuncSetAttribute(dg_stage_kernel<T, N, MODE, MEDIA>,
+    cudaError_t e = cudaFuncSetAttribute(dg_stage_kernel<N, MODE, MEDIA>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L::SMEM_BYTES));
     int nb = 0;
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, dg_stage_kernel<T, N, MODE, MEDIA>,
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, dg_stage_kernel<N, MODE, MEDIA>,
                                                         L::THREADS, L::SMEM_BYTES);
     if (e == cudaSuccess) blocks_per_sm.store(nb > 0 ? nb : 1);
     return e;
@@ -524,29 +500,29 @@ cudaError_t launch_stage_mode(const StageArgs<T>& args, int num_sms, cudaStream_
   int64_t grid = static_cast<int64_t>(blocks_per_sm.load()) * num_sms;
   if (grid > nblk) grid = nblk;
   if (grid < 1) grid = 1;
-  return launch_chained(dg_stage_kernel<T, N, MODE, MEDIA>, static_cast<unsigned>(grid),
+  return launch_chained(dg_stage_kernel<N, MODE, MEDIA>, static_cast<unsigned>(grid),
                         L::THREADS, L::SMEM_BYTES, stream, args);
 }
 
-template <typename T, int N, bool MEDIA>
-cudaError_t launch_stage_any(const StageArgs<T>& args, int mode, int num_sms,
+template <int N, bool MEDIA>
+cudaError_t launch_stage_any(const StageArgs<float>& args, int mode, int num_sms,
                              cudaStream_t stream) {
-  if (mode == kModeRhs) return launch_stage_mode<T, N, kModeRhs, MEDIA>(args, num_sms, stream);
+  if (mode == kModeRhs) return launch_stage_mode<N, kModeRhs, MEDIA>(args, num_sms, stream);
   if (mode == kModeFirstStage)
-    return launch_stage_mode<T, N, kModeFirstStage, MEDIA>(args, num_sms, stream);
-  return launch_stage_mode<T, N, kModeStage, MEDIA>(args, num_sms, stream);
+    return launch_stage_mode<N, kModeFirstStage, MEDIA>(args, num_sms, stream);
+  return launch_stage_mode<N, kModeStage, MEDIA>(args, num_sms, stream);
 }
 
 // Definitions of the launchers declared in launch.h; explicitly instantiated
 // per order in kernels_N*.cu.
-template <typename T, int N>
-cudaError_t launch_stage(const StageArgs<T>& args, int mode, int num_sms, cudaStream_t stream) {
-  return launch_stage_any<T, N, false>(args, mode, num_sms, stream);
+template <int N>
+cudaError_t launch_stage(const StageArgs<float>& args, int mode, int num_sms, cudaStream_t stream) {
+  return launch_stage_any<N, false>(args, mode, num_sms, stream);
 }
-template <typename T, int N>
-cudaError_t launch_stage_media(const StageArgs<T>& args, int mode, int num_sms,
+template <int N>
+cudaError_t launch_stage_media(const StageArgs<float>& args, int mode, int num_sms,
                                cudaStream_t stream) {
-  return launch_stage_any<T, N, true>(args, mode, num_sms, stream);
+  return launch_stage_any<N, true>(args, mode, num_sms, stream);
 }
 
 }  // namespace dgw

@@ -1,10 +1,8 @@
-// Order-3 instantiations of the fused CUDA-core stage kernel (FP32 and
-// FP64; uniform medium and per-element permittivity).
+// Order-3 instantiations of the node-thread FP32 stage kernel (uniform
+// medium and per-element permittivity).
 #include "kernels.cuh"
 
 namespace dgw {
-template cudaError_t launch_stage<float, 3>(const StageArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_stage<double, 3>(const StageArgs<double>&, int, int, cudaStream_t);
-template cudaError_t launch_stage_media<float, 3>(const StageArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_stage_media<double, 3>(const StageArgs<double>&, int, int, cudaStream_t);
+template cudaError_t launch_stage<3>(const StageArgs<float>&, int, int, cudaStream_t);
+template cudaError_t launch_stage_media<3>(const StageArgs<float>&, int, int, cudaStream_t);
 }  // namespace dgw

@@ -46,15 +46,37 @@ __host__ __device__ constexpr bool block_ok(int k0, int n, int E, int64_t fstrid
   return k0 >= 0 && n >= 1 && n <= E && (static_cast<int64_t>(k0) + n) * Np <= fstride;
 }
 
-// Elements per block of the CUDA-core stage kernel (kernels.cuh): a multiple
-// of 4, so every per-block chunk (E Np values, E geometry records, E
+// Elements per block of the node-thread stage kernel (kernels.cuh): a
+// multiple of 4, so every per-block chunk (E Np values, E geometry records, E
 // face-code triples) is a whole number of 16-byte units as TMA requires;
 // E Np <= 512 from N = 4 on, because ptxas budgets registers for the CTA
 // rounded up to 4 warps and each thread needs 2 Np + Nafp registers for its
 // matrix rows.
-__host__ __device__ constexpr int simt_block_elems(int N, bool fp64) {
-  return fp64 ? (N == 1 ? 32 : N <= 4 ? 16 : N == 5 ? 12 : 8)
-              : (N == 1 ? 64 : N <= 4 ? 32 : N == 5 ? 24 : N == 6 ? 16 : 12);
+__host__ __device__ constexpr int simt_block_elems(int N) {
+  return N == 1 ? 64 : N <= 4 ? 32 : N == 5 ? 24 : N == 6 ? 16 : 12;
+}
+
+// FP64 stage kernel (kernels_f64.cuh).  Most elements per block: threads E Np
+// just under a whole number of warps (a partial warp costs the FP64 pipe as
+// much as a full one).  GB300, us per LSRK step, products in FP64 (a thread
+// per node, the form before) / in fixed point: N = 1, K = 180,000 640 / 309;
+// 2, 80,000 631 / 329; 3, 45,000 678 / 308; 4, 45,000 1200 / 406; 5, 101,250
+// 4020 / 1290 (FP64 pipe 0.61 busy by the counter, 0.78 of what back-to-back
+// FMAs reach); 6, 20,000 1267 / 371; 7, 20,000 1965 / 541; with a
+// permittivity 1901 / 560.  Small: N = 4, K = 128 82 / 34; N = 7, K = 128 165
+// / 40.
+__host__ __device__ constexpr int f64_max_elems(int N) {
+  return N == 1 ? 64 : N == 2 ? 16 : N == 3 ? 16 : N == 4 ? 17 : N == 5 ? 9 : N == 6 ? 8 : 7;
+}
+// Elements per block for K elements: fewer than the most where that leaves
+// multiprocessors without a block, but at least 60 threads' worth (the
+// block's table and set-up are its threads' work: N = 7, K = 128, us a step:
+// 77 with one element, 51 with seven).
+inline int f64_block_elems(int N, int64_t K, int num_sms) {
+  const int np = (N + 1) * (N + 2) / 2;
+  const int64_t least = (60 + np - 1) / np, e = (K + num_sms - 1) / num_sms;
+  const int64_t most = f64_max_elems(N);
+  return static_cast<int>(e < least ? least : e < most ? e : most);
 }
 
 // geometry record per element: rx ry sx sy, then per face nx ny Fscale/2
@@ -143,10 +165,10 @@ struct StageArgs {
 
 enum StageMode : int { kModeRhs = 0, kModeFirstStage = 1, kModeStage = 2 };
 
-// One fused stage launch for order N in precision T on the CUDA cores (see
-// kernels.cuh).
-template <typename T, int N>
-cudaError_t launch_stage(const StageArgs<T>& args, int mode, int num_sms, cudaStream_t stream);
+// One fused FP32 stage launch for order N on the CUDA cores, a thread per node
+// (see kernels.cuh).
+template <int N>
+cudaError_t launch_stage(const StageArgs<float>& args, int mode, int num_sms, cudaStream_t stream);
 
 // Tensor-core path (FP32 fields, FP32 accumulation; see kernels_tc.cuh).  The
 // element-local products of a block of elements form one GEMM
@@ -216,6 +238,18 @@ template <int N, int PREC>
 cudaError_t launch_stage_tc(const StageArgs<float>& args, int mode, int num_sms,
                             cudaStream_t stream);
 
+// FP64 path (see kernels_f64.cuh).  tc_op of its StageArgs: Dr and Ds without
+// the vertex nodes' columns, and LIFT, in fixed point -- limb pairs
+// [column][node] of 8 bytes, then per node a pair with the powers of two of
+// its rows' scales (of Dr and Ds, of LIFT); built by f64_operator_table
+// (api.cu).
+__host__ __device__ constexpr int f64_table_pairs(int N) {  // rounded up to 16 bytes
+  return ((2 * (tc_np(N) - 3) + 3 * (N + 1)) * tc_np(N) + 1) / 2 * 2;
+}
+template <int N>
+cudaError_t launch_stage_f64(const StageArgs<double>& args, bool media, int mode, int num_sms,
+                             cudaStream_t stream);
+
 // Element-thread path (FP32, CUDA cores, one thread per element; see
 // kernels_ept.cuh), orders 1..kEptMaxN; the _media launcher takes
 // per-element-permittivity records (kGeoMedia values).  Its reference
@@ -234,9 +268,9 @@ cudaError_t launch_stage_ept_media(const StageArgs<float>& args, const float* op
                                    int num_sms, cudaStream_t stream);
 
 // Operators with a per-element permittivity (geometry records of kGeoMedia
-// values): CUDA-core kernel (FP32 / FP64) and tensor-core kernel (3xTF32).
-template <typename T, int N>
-cudaError_t launch_stage_media(const StageArgs<T>& args, int mode, int num_sms,
+// values): node-thread kernel and tensor-core kernel (3xTF32).
+template <int N>
+cudaError_t launch_stage_media(const StageArgs<float>& args, int mode, int num_sms,
                                cudaStream_t stream);
 template <int N>
 cudaError_t launch_stage_tc_media(const StageArgs<float>& args, int mode, int num_sms,
