@@ -300,7 +300,9 @@ dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, double* ms_tc,
 /* dg_operator_set_block_elems: the element-block size of the operator's
  * kernel for later calls: 0 or the default size, or the tensor-core
  * kernel's alternative size where it has one (3xTF32 products; see
- * dg_operator_tune).  The blocks are a kernel's unit of work: each CTA of
+ * dg_operator_tune).  On a large mesh at N = 3..5 the default is a kernel
+ * with one GEMM row per element and blocks of 128; the sizes of the other
+ * tensor-core kernel (80 and 40, 40 and 80, 40) select that one.  The blocks are a kernel's unit of work: each CTA of
  * the persistent launch walks blocks of this many consecutive elements.
  * Results do not depend on the size beyond rounding.  With face pairs on,
  * the default size is used.

@@ -33,6 +33,7 @@ def _nvcc():
 
 def sources():
     names = (["host_setup.cpp", "api.cu"] + ["kernels_N%d.cu" % n for n in range(1, 8)]
+             + ["kernels_er_N%d.cu" % n for n in range(3, 6)]
              + ["kernels_f64_N%d.cu" % n for n in range(1, 8)]
              + ["kernels_tc_N%d.cu" % n for n in range(1, 8)]
              + ["kernels_tcp_N%d.cu" % n for n in range(1, 8)]

@@ -35,7 +35,8 @@ dg_status cuda_fail(cudaError_t err, const char* where) {
 
 void free_device(dg_op* op) {
   void* ptrs[] = {op->d_Dr,   op->d_Ds,     op->d_LIFT, op->d_geo, op->d_conn,    op->d_qtmp,
-                  op->d_flag, op->d_status, op->d_tcop, op->d_lam, op->d_src_w};
+                  op->d_flag, op->d_status, op->d_tcop, op->d_lam, op->d_src_w, op->d_erop};
+  op->d_erop = nullptr;
   for (void* p : ptrs)
     if (p) cudaFree(p);
   op->d_src_w = nullptr;
@@ -174,6 +175,49 @@ namespace {
 
 using dgw::tc_operator_tiles;
 
+// Operator tiles of the element-row kernel (launch.h), as bytes.
+std::vector<unsigned char> er_operator_tiles(const dgw::RefElement& R, bool media) {
+  const int N = R.N, Np = R.Np, Nfp = N + 1, NI = Np - 3;
+  std::vector<float> out(dgw::er_tile_floats(N, media), 0.f);
+  size_t at = 0;  // first float of the tile in hand
+  auto put = [&](int n, int k, int rows, int kp, double v) {
+    const float hi = tf32_round(v);
+    out[at + dgw::tc_canon(n, k, kp)] = hi;
+    out[at + static_cast<size_t>(rows) * kp + dgw::tc_canon(n, k, kp)] =
+        tf32_round(v - static_cast<double>(hi));
+  };
+  auto node = [&](int c) { return c < N - 1 ? c + 1 : c + 2; };
+  const int np8 = dgw::er_np8(N), nf = dgw::er_nf(N), kz = dgw::er_kz(N), kab = dgw::er_kab(N);
+  for (int n = 0; n < Np; ++n)
+    for (int c = 0; c < NI; ++c) {
+      put(n, c, 2 * np8, kz, R.Dr[n * Np + node(c)]);
+      put(np8 + n, c, 2 * np8, kz, R.Ds[n * Np + node(c)]);
+    }
+  at += 2 * static_cast<size_t>(2 * np8) * kz;
+  const bool one = dgw::er_lift_one(N, media);
+  constexpr int KF = dgw::kErKf;
+  for (int f = 0; f < 3; ++f) {
+    for (int n = 0; n < Np; ++n)
+      for (int j = 0; j < Nfp; ++j) {
+        const double v = R.LIFT[n * 3 * Nfp + f * Nfp + j];
+        if (one)
+          put(f * np8 + n, f * KF + j, dgw::er_nl(N), 3 * KF, v);
+        else
+          put(n, j, nf, KF, v);
+      }
+    if (!one) at += 2 * static_cast<size_t>(nf) * KF;
+  }
+  if (one) at += 2 * static_cast<size_t>(dgw::er_nl(N)) * 3 * KF;
+  for (int n = 0; n < Np; ++n)
+    for (int c = 0; c < NI; ++c) {
+      put(n, 8 * (c / 4) + c % 4, nf, kab, R.Dr[n * Np + node(c)]);
+      put(n, 8 * (c / 4) + 4 + c % 4, nf, kab, R.Ds[n * Np + node(c)]);
+    }
+  std::vector<unsigned char> bytes(out.size() * 4);
+  std::memcpy(bytes.data(), out.data(), bytes.size());
+  return bytes;
+}
+
 // Dr, Ds and LIFT in fixed point for the FP64 kernel (f64_table_pairs,
 // launch.h): v = (hi 2^28 + lo) 2^scale, at most 2^55 in size, with a scale
 // per node for its rows of Dr and Ds and one for its row of LIFT.
@@ -272,6 +316,14 @@ dg_status upload(dg_op* op, const std::vector<double>& rec_in,
     err = cudaMemcpy(op->d_tcop, tiles.data(), tiles.size(), cudaMemcpyHostToDevice);
     if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMemcpy(operator tiles)");
   }
+  if (op->use_er) {
+    op->er_weights.assign(lam.begin(), lam.end());
+    const std::vector<unsigned char> tiles = er_operator_tiles(op->ref, op->media());
+    err = dgw::dev_malloc(&op->d_erop, tiles.size());
+    if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMalloc(operator tiles)");
+    err = cudaMemcpy(op->d_erop, tiles.data(), tiles.size(), cudaMemcpyHostToDevice);
+    if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMemcpy(operator tiles)");
+  }
   err = dgw::dev_malloc(&op->d_status, sizeof(int));
   if (err != cudaSuccess) return cuda_fail(err, "dg_operator_setup: cudaMalloc(status)");
   err = cudaMemset(op->d_status, 0, sizeof(int));
@@ -367,6 +419,25 @@ cudaError_t launch_order_ept(const dg_op* op, const dgw::StageArgs<float>& a, in
   }
 }
 
+// The operator's hot-path calls run the element-row kernel (of an operator
+// on the tensor cores; without face pairs, and with alpha = 1 in a uniform
+// medium).
+bool runs_er(const dg_op* op) {
+  return op->use_er && !op->er_off && op->use_tc && !op->use_ept && !op->tc_alt &&
+         !op->face_pairs && (op->media() || op->alpha == 1.0);
+}
+
+cudaError_t launch_order_er(const dg_op* op, dgw::StageArgs<float> a, int mode, cudaStream_t s) {
+  a.tc_op = op->d_erop;
+  const float* w = op->er_weights.data();
+  switch (op->N) {
+    case 3: return dgw::launch_stage_er<3>(a, w, op->media(), mode, op->num_sms, s);
+    case 4: return dgw::launch_stage_er<4>(a, w, op->media(), mode, op->num_sms, s);
+    case 5: return dgw::launch_stage_er<5>(a, w, op->media(), mode, op->num_sms, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 template <typename T>
 cudaError_t launch_order(const dg_op* op, const dgw::StageArgs<T>& a, int mode, cudaStream_t s) {
   if constexpr (sizeof(T) == 8) {
@@ -381,6 +452,7 @@ cudaError_t launch_order(const dg_op* op, const dgw::StageArgs<T>& a, int mode, 
       default: return cudaErrorInvalidValue;
     }
   } else {
+    if (runs_er(op) && !a.stall_gate) return launch_order_er(op, a, mode, s);
     if (op->media()) return launch_order_media(op, a, mode, s);
     if (op->use_ept) return launch_order_ept(op, a, mode, s);
     if (op->use_tc) return launch_order_tc(op, a, mode, s);
@@ -433,12 +505,17 @@ bool tc_has_alt_n(int N) {
 
 // Elements per block of the kernel the operator runs (alt: the alternative
 // size of the tensor-core kernel).
-int block_elems(const dg_op* op, int alt) {
+int kernel_block_elems(const dg_op* op, int alt) {
   if (op->precision == DG_FP32 && op->use_ept) return 32;
   if (op->precision == DG_FP32 && op->use_tc)
     return 40 * dgw::tc_tiles(op->N, op->tc_prec, alt != 0 && op->tc_prec == dgw::kTcTf32x3);
   if (op->precision == DG_FP64) return dgw::f64_max_elems(op->N);
   return dgw::simt_block_elems(op->N);
+}
+
+// The same with the element-row kernel where the operator runs it.
+int block_elems(const dg_op* op, int alt) {
+  return op->precision == DG_FP32 && runs_er(op) ? dgw::kErElems : kernel_block_elems(op, alt);
 }
 
 dg_status check_device_op(const dg_op* op, const char* where) {
@@ -539,6 +616,19 @@ __global__ void finite_scan_kernel(const float* q32, const double* q64, int64_t 
 // ============================================================ C ABI
 namespace {
 
+// Elements from which an operator runs the element-row kernel: two blocks of
+// 128 for every multiprocessor (2.5 at N = 5 with a permittivity), below which
+// too few of its large blocks are in flight.  GB300, us a step, the other
+// tensor-core kernel / this one: N = 3, K = 20,000 33.2 / 33.0, 39,200 46.0 /
+// 39.9, 180,000 124 / 94, 999,698 595 / 445; N = 4, 20,000 39.0 / 40.0, 39,200
+// 54.5 / 50.0, 80,000 91.5 / 74.4, 665,858 622 / 478 (with a permittivity 617 /
+// 509); N = 5, 20,000 47.1 / 49.2, 39,200 67.6 / 62.0, 101,250 138 / 114,
+// 999,698 1118 / 983 (with a permittivity: 39,200 65.2 / 70.0, 51,842 78.5 /
+// 73.1, 999,698 1101 / 1056).  At N = 6 it measured no faster (523 / 528).
+int64_t er_min_elems(int N, bool media, int num_sms) {
+  return static_cast<int64_t>(num_sms) * dgw::kErElems * (N == 5 && media ? 5 : 4) / 2;
+}
+
 // dg_operator_setup and dg_operator_setup_media; eps NULL: eps = 1.
 dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int32_t precision,
                          int32_t flags, dg_op** out) {
@@ -637,6 +727,9 @@ dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int3
       delete op;
       return cuda_fail(err, "dg_operator_setup: device attribute");
     }
+    op->use_er = precision == DG_FP32 && op->use_tc && !op->use_ept &&
+                 op->tc_prec == dgw::kTcTf32x3 && N >= dgw::kErMinN && N <= dgw::kErMaxN &&
+                 mesh->K >= er_min_elems(N, eps != nullptr, op->num_sms);
     dg_status st = DG_OK;
     try {
       std::vector<double> rec;
@@ -916,9 +1009,13 @@ extern "C" dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems) {
   if (!op) return fail(DG_ERR_ARG, "%s: NULL operator", where);
   const bool alt_ok = op->precision == DG_FP32 && op->use_tc && !op->use_ept &&
                       op->tc_prec == dgw::kTcTf32x3 && tc_has_alt_n(op->N);
-  const int def = block_elems(op, 0), alt = alt_ok ? block_elems(op, 1) : def;
-  if (elems == 0 || elems == def) {
+  const int def = kernel_block_elems(op, 0), alt = alt_ok ? kernel_block_elems(op, 1) : def;
+  if (elems == 0 || (op->use_er && elems == dgw::kErElems)) {
     op->tc_alt = 0;
+    op->er_off = false;
+  } else if (elems == def) {
+    op->tc_alt = 0;
+    op->er_off = true;
   } else if (alt_ok && elems == alt) {
     op->tc_alt = 1;
   } else {

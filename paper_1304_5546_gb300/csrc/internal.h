@@ -129,6 +129,12 @@ struct dg_op {
   int* d_flag = nullptr;   // finiteness scan result
   int* d_status = nullptr; // kernel status word (bounded-wait expiry)
   void* d_tcop = nullptr;  // tensor-core operator tiles for FP32 (see tc_operator_tiles)
+  // FP32 on the element-row kernel: what its setup chose (use_er), unless a
+  // block size of the other tensor-core kernel was asked for (er_off); its
+  // operator tiles and vertex-interpolant weights
+  bool use_er = false, er_off = false;
+  void* d_erop = nullptr;
+  std::vector<float> er_weights;
   bool use_tc = false;     // FP32 products on the tensor cores
   bool use_ept = false;    // FP32: the element-thread kernel (takes precedence over use_tc)
   // FP32 operators of order <= kEptMaxN: the element-thread kernel's

@@ -250,6 +250,35 @@ template <int N>
 cudaError_t launch_stage_f64(const StageArgs<double>& args, bool media, int mode, int num_sms,
                              cudaStream_t stream);
 
+// Element-row path (FP32, 3xTF32 products on the tensor cores, one GEMM row
+// per element; see kernels_er.cuh), orders kErMinN..kErMaxN, alpha = 1 or a
+// permittivity.  tc_op of its StageArgs: the operator tiles, each hi then lo in
+// the layout of tc_canon: [Dr ; Ds] without the vertex nodes' columns (2 er_np8
+// x er_kz: Ds from row er_np8 on); LIFT, as one block-diagonal tile (face f:
+// rows from f er_np8, columns from f kErKf) or face by face (er_nf x kErKf);
+// [Dr | Ds] without the vertex nodes' columns, four of each in turn (er_nf x
+// er_kab); built by er_operator_tiles (api.cu).
+constexpr int kErMinN = 3, kErMaxN = 5, kErElems = 128, kErKf = 8;
+__host__ __device__ constexpr int er_kz(int N) { return (tc_np(N) - 3 + 7) / 8 * 8; }
+__host__ __device__ constexpr int er_kab(int N) { return (tc_np(N) - 3 + 3) / 4 * 8; }
+__host__ __device__ constexpr int er_np8(int N) { return (tc_np(N) + 7) / 8 * 8; }
+__host__ __device__ constexpr int er_nf(int N) { return (tc_np(N) + 15) / 16 * 16; }
+// LIFT as one tile, whose 3 er_np8 accumulator columns (in place of 3 er_nf)
+// leave room for a second accumulator; not at N = 5 with a permittivity, where
+// the larger tile would cost a stage
+__host__ __device__ constexpr bool er_lift_one(int N, bool media) { return !(N == 5 && media); }
+__host__ __device__ constexpr int er_nl(int N) { return (3 * er_np8(N) + 15) / 16 * 16; }
+__host__ __device__ constexpr int er_lift_floats(int N, bool media) {  // hi or lo
+  return er_lift_one(N, media) ? er_nl(N) * 3 * kErKf : 3 * er_nf(N) * kErKf;
+}
+__host__ __device__ constexpr int er_tile_floats(int N, bool media) {
+  return 2 * (2 * er_np8(N) * er_kz(N) + er_lift_floats(N, media) + er_nf(N) * er_kab(N));
+}
+// weights: (1 + r_n) / 2 then (1 + s_n) / 2 at all nodes (host memory)
+template <int N>
+cudaError_t launch_stage_er(const StageArgs<float>& args, const float* weights, bool media,
+                            int mode, int num_sms, cudaStream_t stream);
+
 // Element-thread path (FP32, CUDA cores, one thread per element; see
 // kernels_ept.cuh), orders 1..kEptMaxN; the _media launcher takes
 // per-element-permittivity records (kGeoMedia values).  Its reference
