@@ -209,6 +209,17 @@ __global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
     task_jj[u] = task_j[u] - task_f[u] * Nfp;
   }
 
+  // face codes of the first block's tasks, straight from global memory (no
+  // kernel of the chain writes them): its traces are asked for beside its
+  // stage's copies, not after them
+  int32_t code0[TPT];
+#pragma unroll
+  for (int u = 0; u < TPT; ++u) {
+    const int k = first * E + task_e[u];
+    code0[u] = niter > 0 && task_e[u] < E && k < K
+                   ? __ldg(p.conn + static_cast<int64_t>(k) * 3 + task_f[u])
+                   : -1;
+  }
   chain_wait();
   chain_trigger();
   int issued = 0;  // (thread 0) iterations whose loads were issued
@@ -218,7 +229,7 @@ __global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
 
   // neighbour traces of this thread's flux tasks, one block ahead
   float trc[TPT][3];
-  auto gather = [&](int it) {
+  auto gather = [&](int it, bool at_start) {
     const int s = it % kStages;
     const int32_t* sc =
         reinterpret_cast<const int32_t*>(stages + s * L::STAGE_BYTES + 6 * L::QB + L::GB);
@@ -228,7 +239,7 @@ __global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
       trc[u][0] = trc[u][1] = trc[u][2] = 0.f;
       const int ee = task_e[u];
       if (ee < E && k0 + ee < K) {
-        const int32_t code = sc[ee * 3 + task_f[u]];
+        const int32_t code = at_start ? code0[u] : sc[ee * 3 + task_f[u]];
 #ifdef DGW_DEVICE_CHECKS
         if (!nbr_code_ok(code, p.fstride, Np)) {
           atomicOr(p.status, kStatusIndex);
@@ -246,10 +257,7 @@ __global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
   };
 
   bool ok = true;
-  if (niter > 0) {
-    ok = mbar_wait_bounded(&bars[0], 0, kWaitLimitNs);
-    if (ok) gather(0);
-  }
+  if (niter > 0) gather(0, true);
 
   int it = 0;
   for (; it < niter; ++it) {
@@ -347,7 +355,7 @@ __global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
     if (it + 1 < niter) {
       const uint32_t par1 = static_cast<uint32_t>(((it + 1) / kStages) & 1);
       ok = mbar_wait_bounded(&bars[(it + 1) % kStages], par1, kWaitLimitNs);
-      if (ok) gather(it + 1);
+      if (ok) gather(it + 1, false);
     }
     if (__syncthreads_or(!ok)) break;
     // stage s is no longer read: refill it with block it + kStages

@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(ErLayout<N, MEDIA>::THREADS, 1)
         if (MODE == kModeStage)
           mbar_wait_bounded(&full_r[i % RBAR], static_cast<uint32_t>((i / RBAR) & 1), kWaitLimitNs);
     }
-    bulk_wait_all();
+    bulk_wait_read_all();  // the end of the kernel completes the writes
   } else if (warp == L::MMA_WARP) {
     // ======================= MMA warp (lane 0)
     if (lane == 0) {

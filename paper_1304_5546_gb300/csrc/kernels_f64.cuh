@@ -214,9 +214,6 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
     task_e[u] = tau < E * Nafp ? tau / Nafp : E;  // E: none
     task_j[u] = tau - (tau / Nafp) * Nafp;
   }
-  chain_wait();
-  chain_trigger();
-  if (niter > 0) issue_q(0);
   cp_async_commit();
   cp_async_wait<0>();
   __syncthreads();
@@ -247,7 +244,15 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
       }
     }
   };
-  if (niter > 0) gather(0);
+  chain_wait();
+  chain_trigger();
+  if (niter > 0) {  // the first block's values and traces side by side
+    issue_q(0);
+    cp_async_commit();
+    gather(0);
+    cp_async_wait<0>();
+  }
+  __syncthreads();
 
   for (int it = 0; it < niter; ++it) {
     const int k0 = (b0 + it * G) * E;

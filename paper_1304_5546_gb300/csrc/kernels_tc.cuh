@@ -543,6 +543,26 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
   // launch is not chained, and its memory warp fetches them as it starts
   // (here they measured 1.4 % slower there)
   if (!TABLE && warp == L::IO_WARP && lane == 0 && !p.stall_gate) fetch_tiles();
+  // flux threads: the face codes of the first block's tasks, straight from
+  // global memory (no kernel of the chain writes them), so that its traces are
+  // asked for at once, beside its stage's copies and not after them (a step
+  // at N = 3, K = 1058 24.0 -> 22.9 us, at N = 6, K = 51,842 91.5 -> 89.8; in
+  // the kernels of bf16x3 products and of batches, which have no registers
+  // left for it, 135.6 -> 136.3 at N = 7, K = 49,928 and 0.15 % slower)
+  constexpr bool EARLY = !TABLE && PREC != kTcBf16x3;
+  int32_t code0[EARLY ? TPT : 1];
+  if (EARLY && warp >= L::FLUX_WARP0 && warp < L::MMA_WARP && niter > 0) {
+    int k0, nv;
+    block_at(0, k0, nv);
+#pragma unroll
+    for (int u = 0; u < TPT; ++u) {
+      const int tau = t - 32 * L::FLUX_WARP0 + u * FT;
+      const int ee = tau / Nafp;
+      code0[EARLY ? u : 0] = tau < TASKS && ee < nv
+                     ? __ldg(p.conn + static_cast<int64_t>(k0 + ee) * 3 + (tau - ee * Nafp) / Nfp)
+                     : -1;
+    }
+  }
   if constexpr (!TABLE) {
     chain_wait();
     chain_trigger();
@@ -672,7 +692,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
             mbar_wait_bounded(&full[jj % S], static_cast<uint32_t>((jj / S) & 1), kWaitLimitNs);
         }
       }
-      bulk_wait_all();
+      bulk_wait_read_all();  // the end of the kernel completes the writes
     } else {
       // ======================= memory warp: TMA loads, bulk stores (lane 0)
       if (lane == 0) {
@@ -755,7 +775,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           for (int jj = (issued > S ? issued - S : 0); jj < issued; ++jj)
             mbar_wait_bounded(&full[jj % S], static_cast<uint32_t>((jj / S) & 1), kWaitLimitNs);
         }
-        bulk_wait_all();
+        bulk_wait_read_all();
       }
     }
   } else if (warp == L::MMA_WARP) {
@@ -845,7 +865,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
       task_fo[u] = ee * FES + j;
     }
     float trc[TPT][3];
-    auto gather = [&](int it) {
+    auto gather = [&](int it, bool at_start) {
       const int32_t* sc = reinterpret_cast<const int32_t*>(stages + (it % S) * L::STAGE_BYTES +
                                                            6 * L::QB + L::GB);
       int k0, nv;
@@ -855,7 +875,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
         trc[u][0] = trc[u][1] = trc[u][2] = 0.f;
         const int ee = task_e[u];
         if (ee < nv) {
-          const int32_t code = sc[task_cf[u]];
+          const int32_t code = EARLY && at_start ? code0[EARLY ? u : 0] : sc[task_cf[u]];
 #ifdef DGW_DEVICE_CHECKS
           if (!nbr_code_ok(code, fs, Np)) {
             atomicOr(p.status, kStatusIndex);
@@ -877,8 +897,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
     };
     bool ok = true;
     if (niter > 0) {
-      ok = mbar_wait_or_abort(&full[0], 0, abort_flag);
-      if (ok) gather(0);
+      if (!EARLY) ok = mbar_wait_or_abort(&full[0], 0, abort_flag);
+      if (ok) gather(0, true);
     }
     for (int j = 0; ok && j < niter; ++j) {
       const int s = j % S;
@@ -1005,7 +1025,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
       if (j + 1 < niter) {  // next block's traces, one block ahead
         ok = mbar_wait_or_abort(&full[(j + 1) % S], static_cast<uint32_t>(((j + 1) / S) & 1),
                                 abort_flag);
-        if (ok) gather(j + 1);
+        if (ok) gather(j + 1, false);
       }
     }
     if (!ok) fail();

@@ -157,11 +157,6 @@ __device__ __forceinline__ void bulk_wait_read_all() {
 __device__ __forceinline__ void bulk_wait_read_but_last() {
   asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
 }
-// wait until every committed bulk store has completed
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
 // Per-thread asynchronous copy of 16 bytes global -> shared (L2 only, not
 // cached in L1); both addresses 16-byte aligned.  Completion is tracked per
 // thread in commit groups.
