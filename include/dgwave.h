@@ -163,7 +163,9 @@ void dg_mesh_destroy(dg_mesh* mesh);
  * element-local products (Dr, Ds, LIFT) on the tensor cores as three TF32
  * products per term (hi/lo splits of both operands, FP32 accumulation) from
  * N = 3 on, and on the CUDA cores below, one thread per element (the
- * element-thread kernel).  DG_SETUP_TC selects the
+ * element-thread kernel); on a mesh of a few elements per multiprocessor they
+ * run it on the CUDA cores at every order, one thread per node
+ * (dg_operator_kernel reports the kernel taken).  DG_SETUP_TC selects the
  * tensor cores at every order, DG_SETUP_SIMT the node-thread CUDA-core FP32
  * kernel, DG_SETUP_ELEMENT_THREADS the element-thread kernel (N <= 5), and
  * one of DG_SETUP_TC_TF32 / _BF16 / _BF16X3 a
@@ -228,7 +230,8 @@ dg_status dg_operator_set_alpha(dg_op* op, double alpha);
  * compiler contract multiply-adds).  It applies to the default 3xTF32
  * products; the other product variants, operators on the CUDA-core kernel
  * (FP64, DG_SETUP_SIMT), the element-thread kernel (FP32 at N <= 2 by
- * default, DG_SETUP_ELEMENT_THREADS) and batches ignore it.
+ * default, DG_SETUP_ELEMENT_THREADS) and batches ignore it.  With it on, a
+ * small mesh takes the kernel that it would take if it were larger.
  * Measured slower than the default on GB300 at every order, so off by
  * default.  Errors: DG_ERR_ARG (NULL, enable not 0 or 1).                  */
 dg_status dg_operator_set_face_pairs(dg_op* op, int32_t enable);
@@ -302,8 +305,11 @@ dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, double* ms_tc,
  * kernel's alternative size where it has one (3xTF32 products; see
  * dg_operator_tune).  On a large mesh at N = 3..5 the default is a kernel
  * with one GEMM row per element and blocks of 128; the sizes of the other
- * tensor-core kernel (80 and 40, 40 and 80, 40) select that one.  The blocks are a kernel's unit of work: each CTA of
- * the persistent launch walks blocks of this many consecutive elements.
+ * tensor-core kernel (80 and 40, 40 and 80, 40) select that one; on a small
+ * mesh, where the default is a CUDA-core kernel, they do so too (at N <= 2, 32
+ * selects the element-thread kernel).  The blocks are a kernel's unit of work:
+ * each CTA of the persistent launch walks blocks of this many consecutive
+ * elements.
  * Results do not depend on the size beyond rounding.  With face pairs on,
  * the default size is used.
  * Errors: DG_ERR_ARG (NULL, a size the operator's kernel does not have). */
@@ -311,8 +317,9 @@ dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems);
 
 /* dg_operator_kernel: the kernel the operator's hot-path calls run
  * (DG_KERNEL_*) and its elements per block (the element-thread kernel: 32,
- * one per lane of a warp; the FP64 kernel: the most a block holds, smaller
- * meshes take smaller blocks).  Errors: DG_ERR_ARG (NULL).                */
+ * one per lane of a warp; the FP64 and the node-thread kernel: the most a
+ * block holds, smaller meshes take smaller blocks).  Errors: DG_ERR_ARG
+ * (NULL).                                                                 */
 #define DG_KERNEL_TENSOR_CORES 0
 #define DG_KERNEL_CUDA_CORES 1
 #define DG_KERNEL_ELEMENT_THREADS 2

@@ -390,8 +390,6 @@ cudaError_t launch_order_ept_media(const dg_op* op, const dgw::StageArgs<float>&
 
 cudaError_t launch_order_media(const dg_op* op, const dgw::StageArgs<float>& a, int mode,
                                cudaStream_t s) {
-  if (op->use_ept) return launch_order_ept_media(op, a, mode, s);
-  if (op->use_tc) return launch_order_tc_media(op, a, mode, s);
   switch (op->N) {
     case 1: return dgw::launch_stage_media<1>(a, mode, op->num_sms, s);
     case 2: return dgw::launch_stage_media<2>(a, mode, op->num_sms, s);
@@ -427,6 +425,11 @@ bool runs_er(const dg_op* op) {
          !op->face_pairs && (op->media() || op->alpha == 1.0);
 }
 
+// They run the CUDA-core kernel of small meshes (small_kernel below).
+bool runs_small(const dg_op* op) {
+  return op->small != dgw::kSmallNone && !op->small_off && !op->face_pairs;
+}
+
 cudaError_t launch_order_er(const dg_op* op, dgw::StageArgs<float> a, int mode, cudaStream_t s) {
   a.tc_op = op->d_erop;
   const float* w = op->er_weights.data();
@@ -453,9 +456,12 @@ cudaError_t launch_order(const dg_op* op, const dgw::StageArgs<T>& a, int mode, 
     }
   } else {
     if (runs_er(op) && !a.stall_gate) return launch_order_er(op, a, mode, s);
+    const bool small = runs_small(op) && !a.stall_gate;
+    if (small ? op->small == dgw::kSmallElems : op->use_ept)
+      return op->media() ? launch_order_ept_media(op, a, mode, s) : launch_order_ept(op, a, mode, s);
+    if (op->use_tc && !small)
+      return op->media() ? launch_order_tc_media(op, a, mode, s) : launch_order_tc(op, a, mode, s);
     if (op->media()) return launch_order_media(op, a, mode, s);
-    if (op->use_ept) return launch_order_ept(op, a, mode, s);
-    if (op->use_tc) return launch_order_tc(op, a, mode, s);
     switch (op->N) {
       case 1: return dgw::launch_stage<1>(a, mode, op->num_sms, s);
       case 2: return dgw::launch_stage<2>(a, mode, op->num_sms, s);
@@ -513,8 +519,11 @@ int kernel_block_elems(const dg_op* op, int alt) {
   return dgw::simt_block_elems(op->N);
 }
 
-// The same with the element-row kernel where the operator runs it.
+// The same with the kernels of large and of small meshes where the operator
+// runs them.
 int block_elems(const dg_op* op, int alt) {
+  if (op->precision == DG_FP32 && runs_small(op))
+    return op->small == dgw::kSmallElems ? 32 : dgw::simt_block_elems(op->N);
   return op->precision == DG_FP32 && runs_er(op) ? dgw::kErElems : kernel_block_elems(op, alt);
 }
 
@@ -629,6 +638,29 @@ int64_t er_min_elems(int N, bool media, int num_sms) {
   return static_cast<int64_t>(num_sms) * dgw::kErElems * (N == 5 && media ? 5 : 4) / 2;
 }
 
+// The CUDA-core kernel that an FP32 operator runs below some number of
+// elements, where the caller has not chosen a kernel.  There a step is its
+// five launches' latency: the tensor-core kernel's loads, products and updates
+// are three roles that hand whole blocks of 40 elements on, for the one block
+// each multiprocessor has, and the node-thread kernel does the same for 4 to
+// 32 elements in one role (simt_small_block_elems, launch.h).  The lines lie
+// where it stops being the faster one.  GB300, us a step, the kernel otherwise
+// taken / node threads: N = 1 (element threads), K = 1058 12.6 / 11.0, 4050
+// 13.7 / 11.7, 9800 11.3 / 12.4; N = 2 (element threads), 1058 14.0 / 11.4,
+// 4050 14.9 / 12.7, 9800 14.2 / 15.5; N = 3, 128 26.6 / 11.7, 1058 23.0 / 11.7,
+// 7200 27.1 / 17.9; N = 4, 128 19.9 / 12.2, 1058 22.1 / 13.2, 4802 24.2 / 19.5,
+// 6050 25.9 / 28.7; N = 5, 128 23.6 / 15.2, 2048 24.4 / 19.8, 2450 24.6 / 23.2,
+// 4050 27.4 / 33.5; N = 6, 512 35.4 / 21.4, 1058 29.4 / 22.1, 1568 25.8 / 30.9;
+// N = 7, 512 42.6 / 24.1, 1058 34.7 / 29.8, 1800 30.4 / 36.6 (with a
+// permittivity 800 30.1 / 31.9).  N = 3 above that, tensor cores / element
+// threads: 9800 28.7 / 21.6, 20,000 32.7 / 25.8, 29,768 38.2 / 29.3.
+int small_kernel(int N, bool media, int64_t K, int num_sms) {
+  const int per_sm[8] = {0, 32, 32, 56, 32, 16, 8, media ? 4 : 8};
+  if (K <= static_cast<int64_t>(num_sms) * per_sm[N]) return dgw::kSmallNodes;
+  if (N == 3 && K <= static_cast<int64_t>(num_sms) * 224) return dgw::kSmallElems;
+  return dgw::kSmallNone;
+}
+
 // dg_operator_setup and dg_operator_setup_media; eps NULL: eps = 1.
 dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int32_t precision,
                          int32_t flags, dg_op** out) {
@@ -640,6 +672,8 @@ dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int3
   const int32_t known = DG_SETUP_HOST_ONLY | DG_SETUP_SIMT | DG_SETUP_TC_TF32 | DG_SETUP_TC_BF16 |
                         DG_SETUP_TC_BF16X3 | DG_SETUP_TC | DG_SETUP_ELEMENT_THREADS;
   const int32_t variants = flags & (DG_SETUP_TC_TF32 | DG_SETUP_TC_BF16 | DG_SETUP_TC_BF16X3);
+  const int32_t chosen_kernels = DG_SETUP_SIMT | DG_SETUP_TC | DG_SETUP_TC_TF32 |
+                                 DG_SETUP_TC_BF16 | DG_SETUP_TC_BF16X3;
   if (flags & ~known) return fail(DG_ERR_ARG, "dg_operator_setup: unknown flags 0x%x", flags);
   if ((flags & DG_SETUP_TC) && ((flags & DG_SETUP_SIMT) || precision != DG_FP32))
     return fail(DG_ERR_ARG, "dg_operator_setup: DG_SETUP_TC is for FP32 without DG_SETUP_SIMT");
@@ -672,10 +706,8 @@ dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int3
     // 0.70, 0.86, 1.37; N = 2 0.64, 0.95, 0.82; N = 3 0.64, 0.89, 0.61)
     op->use_tc = (precision == DG_FP32) && !(flags & DG_SETUP_SIMT) &&
                  (N >= 2 || variants != 0 || (flags & DG_SETUP_TC));
-    const int32_t chosen = DG_SETUP_SIMT | DG_SETUP_TC | DG_SETUP_TC_TF32 | DG_SETUP_TC_BF16 |
-                           DG_SETUP_TC_BF16X3;
     op->use_ept = (flags & DG_SETUP_ELEMENT_THREADS) ||
-                  (precision == DG_FP32 && !(flags & chosen) && N <= 2);
+                  (precision == DG_FP32 && !(flags & chosen_kernels) && N <= 2);
     op->tc_prec = (flags & DG_SETUP_TC_TF32)    ? dgw::kTcTf32
                   : (flags & DG_SETUP_TC_BF16)  ? dgw::kTcBf16
                   : (flags & DG_SETUP_TC_BF16X3) ? dgw::kTcBf16x3
@@ -730,6 +762,8 @@ dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int3
     op->use_er = precision == DG_FP32 && op->use_tc && !op->use_ept &&
                  op->tc_prec == dgw::kTcTf32x3 && N >= dgw::kErMinN && N <= dgw::kErMaxN &&
                  mesh->K >= er_min_elems(N, eps != nullptr, op->num_sms);
+    if (precision == DG_FP32 && !(flags & (chosen_kernels | DG_SETUP_ELEMENT_THREADS)))
+      op->small = small_kernel(N, eps != nullptr, mesh->K, op->num_sms);
     dg_status st = DG_OK;
     try {
       std::vector<double> rec;
@@ -956,7 +990,8 @@ extern "C" dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, dou
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   const bool was_tc = op->use_tc, was_ept = op->use_ept;
-  const int was_alt = op->tc_alt;
+  const int was_alt = op->tc_alt, was_small = op->small;
+  op->small = dgw::kSmallNone;  // its kernels are among the candidates
   float ms[4] = {0.f, 0.f, 0.f, 0.f};
   for (int v = 0; v < nc && err == cudaSuccess; ++v) {
     op->use_tc = cand[v].tc;
@@ -985,6 +1020,7 @@ extern "C" dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, dou
     op->use_tc = was_tc;
     op->tc_alt = was_alt;
     op->use_ept = was_ept;
+    op->small = was_small;
     return cuda_fail(err, "dg_operator_tune");
   }
   int best = 0;
@@ -1012,12 +1048,13 @@ extern "C" dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems) {
   const int def = kernel_block_elems(op, 0), alt = alt_ok ? kernel_block_elems(op, 1) : def;
   if (elems == 0 || (op->use_er && elems == dgw::kErElems)) {
     op->tc_alt = 0;
-    op->er_off = false;
+    op->er_off = op->small_off = false;
   } else if (elems == def) {
     op->tc_alt = 0;
-    op->er_off = true;
+    op->er_off = op->small_off = true;
   } else if (alt_ok && elems == alt) {
     op->tc_alt = 1;
+    op->small_off = true;
   } else {
     return fail(DG_ERR_ARG, "%s: %d elements per block is not a size of this operator's kernel "
                 "(%d%s%s)", where, elems, def, alt_ok ? " or " : "",
@@ -1029,8 +1066,9 @@ extern "C" dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems) {
 extern "C" dg_status dg_operator_kernel(const dg_op* op, int32_t* kernel, int32_t* elems) {
   dgw::clear_error();
   if (!op) return fail(DG_ERR_ARG, "dg_operator_kernel: NULL operator");
-  const bool ept = op->precision == DG_FP32 && op->use_ept;
-  const bool tc = op->precision == DG_FP32 && op->use_tc && !ept;
+  const bool fp32 = op->precision == DG_FP32, small = fp32 && runs_small(op);
+  const bool ept = small ? op->small == dgw::kSmallElems : fp32 && op->use_ept;
+  const bool tc = fp32 && op->use_tc && !ept && !small;
   if (kernel)
     *kernel = ept ? DG_KERNEL_ELEMENT_THREADS : tc ? DG_KERNEL_TENSOR_CORES : DG_KERNEL_CUDA_CORES;
   if (elems) *elems = block_elems(op, op->tc_alt && !op->face_pairs);
@@ -1333,7 +1371,7 @@ extern "C" dg_status dg_test_wait_timeout(const dg_op* op, void* stream) {
   if (err == cudaSuccess) err = cudaMemsetAsync(gate, 0, sizeof(int), s);
   if (err == cudaSuccess) {
     dgw::StageArgs<float> a = base_args<float>(op);
-    a.qin = static_cast<const float*>(op->d_qtmp);  // never read: the wait runs out first
+    a.qin = static_cast<const float*>(op->d_qtmp);  // values unused: the wait runs out first
     a.rhs = static_cast<float*>(op->d_qtmp);
     a.stall_gate = gate;
     err = launch_order<float>(op, a, dgw::kModeRhs, s);

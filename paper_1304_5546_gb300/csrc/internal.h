@@ -133,6 +133,10 @@ struct dg_op {
   // block size of the other tensor-core kernel was asked for (er_off); its
   // operator tiles and vertex-interpolant weights
   bool use_er = false, er_off = false;
+  // FP32 on a small mesh: the kernel its setup chose instead (kSmall...),
+  // unless a block size of the kernel below was asked for (small_off)
+  int small = 0;
+  bool small_off = false;
   void* d_erop = nullptr;
   std::vector<float> er_weights;
   bool use_tc = false;     // FP32 products on the tensor cores

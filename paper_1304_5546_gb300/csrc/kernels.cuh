@@ -56,13 +56,13 @@ constexpr int kStages = 3;
 
 constexpr int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-template <int N, bool MEDIA = false>
+template <int N, bool MEDIA, int E_>
 struct Layout {
   static constexpr int GEO = MEDIA ? kGeoMedia : kGeo;  // geometry record length
   static constexpr int Np = Order<N>::Np;
   static constexpr int Nfp = Order<N>::Nfp;
   static constexpr int Nafp = Order<N>::Nafp;
-  static constexpr int E = simt_block_elems(N);
+  static constexpr int E = E_;
   static constexpr int VW = 4;
   static constexpr int NPAD = round_up(Np, VW);
   static constexpr int FPAD = round_up(Nafp, VW);
@@ -124,10 +124,10 @@ cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned threads
 // records of kGeoMedia values (per-element permittivity, see launch.h): the
 // flux of the exact interface Riemann solution and per-row scales of the
 // right-hand side.
-template <int N, int MODE, bool MEDIA>
-__global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
+template <int N, int MODE, bool MEDIA, int E_>
+__global__ void __launch_bounds__(Layout<N, MEDIA, E_>::THREADS)
     dg_stage_kernel(const StageArgs<float> p) {
-  using L = Layout<N, MEDIA>;
+  using L = Layout<N, MEDIA, E_>;
   constexpr int GEO = L::GEO;
   constexpr int Np = L::Np, Nfp = L::Nfp, Nafp = L::Nafp;
   constexpr int E = L::E, NPAD = L::NPAD, FPAD = L::FPAD, VW = L::VW;
@@ -485,20 +485,20 @@ __global__ void __launch_bounds__(Layout<N, MEDIA>::THREADS)
   }
 }
 
-template <int N, int MODE, bool MEDIA>
-cudaError_t launch_stage_mode(const StageArgs<float>& args, int num_sms, cudaStream_t stream) {
-  using L = Layout<N, MEDIA>;
-  // per (N, MODE, MEDIA): shared-memory attribute and resident CTAs per
+template <int N, int MODE, bool MEDIA, int E>
+cudaError_t launch_stage_blocks(const StageArgs<float>& args, int num_sms, cudaStream_t stream) {
+  using L = Layout<N, MEDIA, E>;
+  // per (N, MODE, MEDIA, E): shared-memory attribute and resident CTAs per
   // SM, set on the first launch on each device
   static std::atomic<uint64_t> configured{0};
   static std::atomic<int> blocks_per_sm{1};
   cudaError_t err = configure_once_per_device(configured, [] {
-    cudaError_t e = cudaFuncSetAttribute(dg_stage_kernel<N, MODE, MEDIA>,
+    cudaError_t e = cudaFuncSetAttribute(dg_stage_kernel<N, MODE, MEDIA, E>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(L::SMEM_BYTES));
     int nb = 0;
     if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, dg_stage_kernel<N, MODE, MEDIA>,
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, dg_stage_kernel<N, MODE, MEDIA, E>,
                                                         L::THREADS, L::SMEM_BYTES);
     if (e == cudaSuccess) blocks_per_sm.store(nb > 0 ? nb : 1);
     return e;
@@ -508,8 +508,17 @@ cudaError_t launch_stage_mode(const StageArgs<float>& args, int num_sms, cudaStr
   int64_t grid = static_cast<int64_t>(blocks_per_sm.load()) * num_sms;
   if (grid > nblk) grid = nblk;
   if (grid < 1) grid = 1;
-  return launch_chained(dg_stage_kernel<N, MODE, MEDIA>, static_cast<unsigned>(grid),
+  return launch_chained(dg_stage_kernel<N, MODE, MEDIA, E>, static_cast<unsigned>(grid),
                         L::THREADS, L::SMEM_BYTES, stream, args);
+}
+
+// blocks of the usual size, or of a few elements on a small mesh (launch.h)
+template <int N, int MODE, bool MEDIA>
+cudaError_t launch_stage_mode(const StageArgs<float>& args, int num_sms, cudaStream_t stream) {
+  constexpr int E = simt_block_elems(N), ES = simt_small_block_elems(N);
+  return args.K < static_cast<int64_t>(simt_small_per_sm(N)) * num_sms
+             ? launch_stage_blocks<N, MODE, MEDIA, ES>(args, num_sms, stream)
+             : launch_stage_blocks<N, MODE, MEDIA, E>(args, num_sms, stream);
 }
 
 template <int N, bool MEDIA>

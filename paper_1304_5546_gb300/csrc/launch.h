@@ -55,6 +55,24 @@ __host__ __device__ constexpr bool block_ok(int k0, int n, int E, int64_t fstrid
 __host__ __device__ constexpr int simt_block_elems(int N) {
   return N == 1 ? 64 : N <= 4 ? 32 : N == 5 ? 24 : N == 6 ? 16 : 12;
 }
+// The same on meshes below simt_small_per_sm(N) elements per multiprocessor.
+// There a step's time is that of one block's chain of products and updates,
+// which grows with the block, and most multiprocessors have no block of the
+// usual size.  GB300, us a step, usual / small blocks: N = 1, K = 1058 12.6 /
+// 10.7, 4050 12.7 / 11.3; N = 3, 512 14.3 / 11.6, 2450 14.3 / 12.5, 4050 14.5 /
+// 15.0; N = 4, 512 19.2 / 12.3, 2450 19.3 / 16.7, 4050 19.4 / 20.9; N = 5, 512
+// 25.4 / 15.4, 2450 25.9 / 23.2, 4050 34.2 / 33.6; N = 6, 512 32.6 / 21.4, 1058
+// 33.0 / 22.1, 2450 40.8 / 39.5; N = 7, 512 47.5 / 24.1, 1058 47.1 / 29.8.  4
+// elements measured no better over the range at N = 3..5 (N = 4, 2450: 16.9),
+// 8 at N = 7 worse (512: 32.7).
+__host__ __device__ constexpr int simt_small_block_elems(int N) {
+  return N <= 2 ? 16 : N <= 6 ? 8 : 4;
+}
+__host__ __device__ constexpr int simt_small_per_sm(int N) {
+  return simt_block_elems(N) < 24 ? simt_block_elems(N) : 24;
+}
+// Kernels that an FP32 operator takes on a small mesh (dg_op::small).
+constexpr int kSmallNone = 0, kSmallNodes = 1, kSmallElems = 2;
 
 // FP64 stage kernel (kernels_f64.cuh).  Most elements per block: threads E Np
 // just under a whole number of warps (a partial warp costs the FP64 pipe as

@@ -297,6 +297,8 @@ dg_status build_device(dg_partition& pt) {
     s->tc_prec = op.tc_prec;
     s->use_er = op.use_er;  // the same kernel whatever the part's size: results equal bit for bit
     s->er_off = op.er_off;
+    s->small = op.small;
+    s->small_off = op.small_off;
     s->elem_size = op.elem_size;
     s->device = op.device;
     s->num_sms = op.num_sms;
