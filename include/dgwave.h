@@ -436,9 +436,9 @@ dg_status dg_step_static(const dg_op* op, void* d_q, void* d_res, double t0, dou
 
 /* ------------------------------------------------------------ batches ---
  * A batch steps many independent problems of mixed orders together: each
- * LSRK stage of every problem in the batch is ONE persistent launch (all
- * orders at once; the launch's CTAs are split among the orders), and a step
- * (five stages) is replayed from a captured CUDA graph.  Problems join and
+ * LSRK stage of every problem of an order is ONE persistent launch (or of
+ * all orders at once; see the launch modes), and a step (five stages) of
+ * orders side by side is replayed from a captured CUDA graph.  Problems join and
  * leave between steps (continuous batching); each keeps its own time step.
  * Computation: FP32 fields, tensor-core 3xTF32 products, the per-element
  * permittivity flux of dg_operator_setup_media (eps = 1 for operators set
@@ -462,10 +462,12 @@ dg_status dg_step_static(const dg_op* op, void* d_q, void* d_res, double t0, dou
                                only (see below)                            */
 
 /* Launch modes.  Concurrent (the default): each order's share of a stage
- * is a kernel of its own with one CTA per SM over that order's blocks; the
- * orders' kernels run side by side on streams of the batch, joined once per
- * step, and the hardware hands SMs to whichever order has CTAs waiting, so
- * orders do not wait for each other at every stage.  Split (DG_BATCH_SPLIT,
+ * is a kernel of its own with one CTA per SM over that order's blocks.  An
+ * order whose blocks fill the SMs runs by itself, the steps of a call as one
+ * chain of launches on the caller's stream; the others' kernels run side by
+ * side on streams of the batch, joined once per step, and the hardware hands
+ * SMs to whichever order has CTAs waiting, so orders do not wait for each
+ * other at every stage.  Split (DG_BATCH_SPLIT,
  * or when dg_batch_tune measures it faster): one launch per stage over all
  * orders, its CTAs split among the orders by the planner.                  */
 /* dg_batch_create: capacity[N-1] = elements of order N the batch can hold
@@ -515,7 +517,8 @@ dg_status dg_batch_get_fields(dg_batch* batch, int32_t slot, void* dst, int64_t 
                               void* stream);
 
 /* dg_batch_step: nsteps LSRK(5,4) steps of every problem in the batch, each
- * with its own dt; per stage one launch over all problems.  The first call
+ * with its own dt; per stage one launch over all problems (of an order, or of
+ * all orders; see the launch modes).  The first call
  * after a problem joined or left uploads the block tables and CTA split
  * (asynchronously on `stream`).  Calls on one batch must be ordered (one
  * stream, or the caller's synchronisation).  Unless DG_BATCH_NO_ADAPT, the

@@ -709,7 +709,7 @@ class Batch:
     ``capacity``: dict order -> element capacity, or 7 counts.  ``add``
     admits a Solver's operator (FP32) with its time step; fields move in and
     out as (3, K, Np) arrays.  ``split``: the split launch mode only
-    (DG_BATCH_SPLIT); by default the orders' kernels run side by side.
+    (DG_BATCH_SPLIT); by default each order has kernels of its own.
     """
 
     def __init__(self, capacity, graph=True, adapt=True, device=None, split=False):

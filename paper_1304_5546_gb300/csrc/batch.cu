@@ -13,9 +13,9 @@
 // A launch walks a block table per order (E-element blocks that never span
 // two problems; the last block of a problem may be short).  Tables, block
 // counts and the split of the launch's CTAs among the orders live in device
-// memory and are rewritten when problems join or leave, so the two captured
-// one-step graphs (starting from either ping-pong buffer) stay valid for the
-// batch's lifetime.
+// memory and are rewritten when problems join or leave, so the captured
+// one-step graphs (one from either ping-pong buffer, for each set of orders
+// that run side by side) stay valid.
 //
 // The CTA split: order N's blocks take ceil(nblk_N / c_N) iterations of
 // tau_N seconds on each of its c_N CTAs; the planner gives every order with
@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
 #include <map>
@@ -43,6 +44,7 @@ using dgw::fail;
 namespace {
 
 constexpr int kOrders = DG_N_MAX;
+constexpr size_t kMaxGraphs = 8;  // sets of orders whose step graphs are kept
 constexpr int kPadElems = 8;  // pool tail read by the last block's 16-byte rounding
 
 dg_status cuda_fail(cudaError_t err, const char* where) {
@@ -83,26 +85,31 @@ struct dg_batch {
   int flags = 0;
   Pool pools[kOrders];
   int* d_meta = nullptr;  // [0, 7): block counts per order, [8, 16): CTA split cta0,
-                          // [16]: steps completed (stage time of the point sources)
+                          // [16, 23): steps completed, per order (stage time of the point
+                          // sources)
   int* d_status = nullptr;
   // point sources, indexed by problem slot
   int64_t max_slots = 0;
   float* d_src_w = nullptr;      // [slot][kSrcStride]
   double* d_src_meta = nullptr;  // [slot][4]: dt, t0, pi f, amplitude
   int* d_src_step = nullptr;     // [slot]: steps enqueued when the problem joined
-  int64_t steps = 0;             // steps enqueued so far
+  int64_t steps[kOrders] = {};   // steps enqueued so far, per order (the device counters)
   std::vector<Problem> probs;
   int cur = 0;  // ping-pong buffer holding the current fields
   bool dirty = true;
   int64_t nblk[kOrders] = {};
+  bool alone[kOrders] = {};  // concurrent mode: the order runs by itself (plan_sequence)
   int cta[kOrders] = {};
   double cost[kOrders] = {};  // seconds (or model units) per block iteration of one CTA
   bool measured = false;
   size_t smem = 0;
-  cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  // one step's launches, by source buffer, for each set of orders that ran
+  // side by side (side_by_side; the split mode: set 0)
+  std::map<unsigned, std::array<cudaGraphExec_t, 2>> graphs;
   cudaStream_t capture = nullptr;
-  // launch mode: concurrent (each order's stage a kernel of its own, the
-  // orders side by side on streams of their own, joined once per step) or,
+  // launch mode: concurrent (each order's stage a kernel of its own; orders
+  // by themselves, or side by side on streams of their own, joined once per
+  // step) or,
   // with DG_BATCH_SPLIT or when dg_batch_tune measures it faster, split (one
   // launch per stage, its CTAs split among the orders)
   bool concurrent = true;
@@ -173,6 +180,13 @@ double model_cost(int N) {
   return 1e-6 * us[N];
 }
 
+void drop_graphs(dg_batch* b) {
+  for (auto& gs : b->graphs)
+    for (cudaGraphExec_t ge : gs.second)
+      if (ge) cudaGraphExecDestroy(ge);
+  b->graphs.clear();
+}
+
 void free_pool(Pool& p) {
   void* ptrs[] = {p.q[0], p.q[1], p.res, p.geo, p.conn, p.lam, p.tcop, p.blocks};
   for (void* x : ptrs)
@@ -187,8 +201,7 @@ void destroy_batch(dg_batch* b) {
   if (!b) return;
   cudaSetDevice(b->device);
   cudaDeviceSynchronize();
-  for (cudaGraphExec_t& g : b->graph)
-    if (g) cudaGraphExecDestroy(g);
+  drop_graphs(b);
   if (b->capture) cudaStreamDestroy(b->capture);
   for (int g = 0; g < kOrders; ++g) {
     if (b->ostream[g]) cudaStreamDestroy(b->ostream[g]);
@@ -308,20 +321,20 @@ dgw::BatchArgs batch_args(const dg_batch* b, int src, int stage) {
     s.src_w = b->d_src_w;
     s.src_meta = b->d_src_meta;
     s.src_step = b->d_src_step;
-    s.step_ctr = b->d_meta + 16;
+    s.step_ctr = b->d_meta + 16 + g;
     s.c_stage = b->lsrk_c[stage];
   }
   a.cta0 = b->d_meta + 8;
   return a;
 }
 
-// end of a step: the device step counter that the source times read
-__global__ void batch_tick_kernel(int* ctr) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) *ctr += 1;
+// the device step counters, one an order, that the source times read
+__global__ void batch_tick_kernel(int* ctr, unsigned mask, int nsteps) {
+  if (threadIdx.x < kOrders && (mask >> threadIdx.x & 1)) ctr[threadIdx.x] += nsteps;
 }
 
-cudaError_t launch_tick(dg_batch* b, cudaStream_t s) {
-  batch_tick_kernel<<<1, 32, 0, s>>>(b->d_meta + 16);
+cudaError_t launch_tick(dg_batch* b, unsigned mask, int nsteps, cudaStream_t s) {
+  batch_tick_kernel<<<1, 32, 0, s>>>(b->d_meta + 16, mask, nsteps);
   cudaError_t err = cudaGetLastError();
   if (err == cudaSuccess) ++b->launches;
   return err;
@@ -337,21 +350,25 @@ cudaError_t launch_stage(dg_batch* b, int src, int stage, cudaStream_t s) {
 }
 
 // Order g's kernel of the concurrent mode for stage `stage`, reading field
-// buffer src; grid 0 only configures the kernel.
-cudaError_t launch_order_stage(dg_batch* b, int g, int src, int stage, int grid, cudaStream_t s) {
-  const dgw::BatchArgs a = batch_args(b, src, stage);
-  const dgw::StageArgs<float>& ga = a.g[g];
+// buffer src; grid 0 only configures the kernel.  chained: behind a launch of
+// the same chain (launch_chained).  The step is the device counter plus
+// step_off.
+cudaError_t launch_order_stage(dg_batch* b, int g, int src, int stage, int grid, cudaStream_t s,
+                               bool chained = false, int step_off = 0) {
+  dgw::BatchArgs a = batch_args(b, src, stage);
+  dgw::StageArgs<float>& ga = a.g[g];
+  ga.step_off = step_off;
   const bool first = stage == 0;
   cudaError_t err = cudaErrorInvalidValue;
   const bool alt = b->pools[g].alt;
 #define DG_ORDER_CASE(NN_)                                                                 \
   case NN_:                                                                                \
     if (alt)                                                                               \
-      err = first ? dgw::launch_batch_order<NN_, dgw::kModeFirstStage, true>(ga, grid, s)  \
-                  : dgw::launch_batch_order<NN_, dgw::kModeStage, true>(ga, grid, s);      \
+      err = first ? dgw::launch_batch_order<NN_, dgw::kModeFirstStage, true>(ga, grid, chained, s)  \
+                  : dgw::launch_batch_order<NN_, dgw::kModeStage, true>(ga, grid, chained, s);      \
     else                                                                                   \
-      err = first ? dgw::launch_batch_order<NN_, dgw::kModeFirstStage>(ga, grid, s)        \
-                  : dgw::launch_batch_order<NN_, dgw::kModeStage>(ga, grid, s);            \
+      err = first ? dgw::launch_batch_order<NN_, dgw::kModeFirstStage>(ga, grid, chained, s)        \
+                  : dgw::launch_batch_order<NN_, dgw::kModeStage>(ga, grid, chained, s);            \
     break;
   switch (g + 1) {
     DG_ORDER_CASE(1)
@@ -369,13 +386,50 @@ cudaError_t launch_order_stage(dg_batch* b, int g, int src, int stage, int grid,
   return err;
 }
 
-// `reps` launches of stage `stage` (reading buffer src) of every order with
-// a pool, each order on its own stream, forked from and joined back into s.
+// Concurrent mode: an order runs by itself, all the steps of a call in one
+// chain of launches (launch_order_steps), when its blocks fill the
+// multiprocessors, and beside the other orders (launch_concurrent) when they
+// do not.  By itself its fields stay in L2 from stage to stage and its launches
+// follow each other in 0.7 us; side by side a stage's tail is filled by another
+// order's blocks.  GB300, us a stage, side by side / by themselves: orders 3, 5
+// and 7 with 9.1, 6.5 and 11.1 blocks per multiprocessor 83.2 / 67.5; 1 to 4
+// with 1.0 to 1.8 33.1 / 27.3; 2, 4 and 6 with 1.2, 2.1 and 2.2 26.5 / 24.1; 3
+// to 7 with 1.6 to 4.0 (a server, ms in all) 15.7 / 15.3; but 1 and 2 with 1.3
+// and 0.3 11.0 / 12.5, 3 and 5 with 0.7 and 1.7 (ms in all) 1.88 / 2.10: where
+// one order cannot fill the machine the others run beside it, unless they have
+// blocks for several rounds.
+void plan_sequence(dg_batch* b) {
+  bool all = true;
+  for (int g = 0; g < kOrders; ++g)
+    all = all && (b->nblk[g] == 0 || b->nblk[g] >= b->num_sms);
+  for (int g = 0; g < kOrders; ++g)
+    b->alone[g] = b->nblk[g] >= (all ? 1 : 4) * static_cast<int64_t>(b->num_sms);
+}
+
+bool in_sequence(const dg_batch* b, int g) { return b->concurrent && b->alone[g]; }
+
+// The other orders with blocks, as a bit mask.
+unsigned side_by_side(const dg_batch* b) {
+  unsigned mask = 0;
+  for (int g = 0; g < kOrders; ++g)
+    if (b->nblk[g] > 0 && !in_sequence(b, g)) mask |= 1u << g;
+  return mask;
+}
+
+// The orders whose step counters launch_step advances.
+unsigned ticked(const dg_batch* b) {
+  return b->concurrent ? side_by_side(b) : (1u << kOrders) - 1;
+}
+
+// `reps` launches of stage `stage` (reading buffer src), or a whole step, of
+// every order of `mask`, each order on its own stream, forked from and joined
+// back into s.
 cudaError_t launch_concurrent(dg_batch* b, int src, int stage, int reps, bool whole_step,
-                              cudaStream_t s) {
+                              unsigned mask, cudaStream_t s) {
+  if (mask == 0) return cudaSuccess;
   cudaError_t err = cudaEventRecord(b->fork_ev, s);
   for (int g = 0; g < kOrders && err == cudaSuccess; ++g) {
-    if (b->pools[g].cap == 0) continue;
+    if (!(mask >> g & 1)) continue;
     err = cudaStreamWaitEvent(b->ostream[g], b->fork_ev, 0);
     if (whole_step) {
       for (int i = 0; i < 5 && err == cudaSuccess; ++i)
@@ -390,16 +444,36 @@ cudaError_t launch_concurrent(dg_batch* b, int src, int stage, int reps, bool wh
   return err;
 }
 
-// One LSRK step of every problem, from field buffer src, in the batch's
-// launch mode, followed by the step-counter tick.
+// `count` launches of stage `stage` (reading buffer src) of order g on s, a
+// chain: each launch has a block for every CTA, so that each waits for the
+// launch before it.
+cudaError_t launch_chain(dg_batch* b, int g, int src, int stage, int count, cudaStream_t s) {
+  cudaError_t err = cudaSuccess;
+  for (int r = 0; r < count && err == cudaSuccess; ++r)
+    err = launch_order_stage(b, g, src, stage, b->num_sms, s, r > 0);
+  return err;
+}
+
+// `count` steps of order g on s from buffer src, a chain of launches behind
+// the tick that takes the order's step counter past them.
+cudaError_t launch_order_steps(dg_batch* b, int g, int src, int count, cudaStream_t s) {
+  cudaError_t err = launch_tick(b, 1u << g, count, s);
+  for (int r = 0; r < 5 * count && err == cudaSuccess; ++r)
+    err = launch_order_stage(b, g, src ^ (r & 1), r % 5, b->num_sms, s, r > 0, r / 5 - count);
+  return err;
+}
+
+// One LSRK step of every problem but those of the orders in_sequence, from
+// field buffer src, in the batch's launch mode, followed by the step-counter
+// tick.
 cudaError_t launch_step(dg_batch* b, int src, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
   if (b->concurrent) {
-    err = launch_concurrent(b, src, 0, 1, true, s);
+    err = launch_concurrent(b, src, 0, 1, true, side_by_side(b), s);
   } else {
     for (int i = 0; i < 5 && err == cudaSuccess; ++i) err = launch_stage(b, src ^ (i & 1), i, s);
   }
-  if (err == cudaSuccess) err = launch_tick(b, s);
+  if (err == cudaSuccess) err = launch_tick(b, ticked(b), 1, s);
   return err;
 }
 
@@ -419,6 +493,7 @@ dg_status upload_tables(dg_batch* b, cudaStream_t s) {
     std::sort(tab[g].begin(), tab[g].end(), [](const int2& x, const int2& y) { return x.x < y.x; });
     b->nblk[g] = static_cast<int64_t>(tab[g].size());
   }
+  plan_sequence(b);
   if (!plan_ctas(b->nblk, b->cost, b->num_sms, b->cta))
     return fail(DG_ERR_ARG, "dg_batch_step: more orders with problems than CTAs");
   size_t total = 0;
@@ -450,7 +525,8 @@ dg_status upload_tables(dg_batch* b, cudaStream_t s) {
   return DG_OK;
 }
 
-dg_status capture_graphs(dg_batch* b) {
+dg_status capture_graphs(dg_batch* b, unsigned set) {
+  if (b->graphs.size() >= kMaxGraphs) drop_graphs(b);
   if (!b->capture) {
     cudaError_t err = cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking);
     if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: stream");
@@ -466,18 +542,26 @@ dg_status capture_graphs(dg_batch* b) {
     if (cerr == cudaSuccess) cerr = launch_order_stage(b, g, 0, 1, 0, b->capture);
   }
   if (cerr != cudaSuccess) return cuda_fail(cerr, "dg_batch_step: kernel attributes");
+  std::array<cudaGraphExec_t, 2>& exec = b->graphs[set];
+  exec = {nullptr, nullptr};
   for (int src = 0; src < 2; ++src) {
     cudaGraph_t graph = nullptr;
     cudaError_t err = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
-    if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: begin capture");
+    if (err != cudaSuccess) {
+      drop_graphs(b);
+      return cuda_fail(err, "dg_batch_step: begin capture");
+    }
     const int64_t before = b->launches;
     const cudaError_t lerr = launch_step(b, src, b->capture);
     b->launches = before;  // captured, not run
     err = cudaStreamEndCapture(b->capture, &graph);
     if (lerr != cudaSuccess) err = lerr;
-    if (err == cudaSuccess) err = cudaGraphInstantiate(&b->graph[src], graph, 0);
+    if (err == cudaSuccess) err = cudaGraphInstantiate(&exec[src], graph, 0);
     if (graph) cudaGraphDestroy(graph);
-    if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: graph capture");
+    if (err != cudaSuccess) {
+      drop_graphs(b);
+      return cuda_fail(err, "dg_batch_step: graph capture");
+    }
   }
   return DG_OK;
 }
@@ -491,17 +575,14 @@ void set_order_alt(dg_batch* b, int g, bool alt) {
   p.alt = alt;
   p.E = dgw::batch_tc_block_elems(g + 1, alt);
   b->dirty = true;
-  for (cudaGraphExec_t& ge : b->graph) {
-    if (ge) cudaGraphExecDestroy(ge);
-    ge = nullptr;
-  }
+  drop_graphs(b);
 }
 
-// kernel launches of one step in the batch's mode (stages and the tick)
+// kernel launches of launch_step (stages and the tick)
 int64_t launches_per_step(const dg_batch* b) {
   if (!b->concurrent) return 6;
   int64_t n = 1;
-  for (int g = 0; g < kOrders; ++g) n += b->pools[g].cap > 0 ? 5 : 0;
+  for (unsigned mask = side_by_side(b); mask; mask &= mask - 1) n += 5;
   return n;
 }
 
@@ -569,8 +650,8 @@ extern "C" dg_status dg_batch_create(const int64_t* capacity, int32_t flags, dg_
     b->cost[g] = model_cost(g + 1);
   }
   for (int g = 0; g < kOrders; ++g) b->max_slots += capacity[g] > 0 ? capacity[g] / 4 + 1 : 0;
-  err = dgw::dev_malloc(reinterpret_cast<void**>(&b->d_meta), 17 * sizeof(int));
-  if (err == cudaSuccess) err = cudaMemset(b->d_meta, 0, 17 * sizeof(int));
+  err = dgw::dev_malloc(reinterpret_cast<void**>(&b->d_meta), 23 * sizeof(int));
+  if (err == cudaSuccess) err = cudaMemset(b->d_meta, 0, 23 * sizeof(int));
   if (err == cudaSuccess)
     err = dgw::dev_malloc(reinterpret_cast<void**>(&b->d_src_w), b->max_slots * dgw::kSrcStride * 4);
   if (err == cudaSuccess)
@@ -677,7 +758,7 @@ extern "C" dg_status dg_batch_add(dg_batch* b, const dg_op* op, double dt,
     hm[3] = src->amplitude;
     for (int n = 0; n < dgw::kSrcStride; ++n)
       hw[n] = n < op->Np ? static_cast<float>(dt * src_wt[n]) : 0.0f;
-    *hs = static_cast<int>(b->steps);
+    *hs = static_cast<int>(b->steps[op->N - 1]);
     err = cudaMemcpyAsync(b->d_src_meta + 4 * id, hm, 4 * sizeof(double), cudaMemcpyHostToDevice, s);
     if (err == cudaSuccess)
       err = cudaMemcpyAsync(b->d_src_w + dgw::kSrcStride * id, hw, dgw::kSrcStride * 4,
@@ -860,19 +941,29 @@ extern "C" dg_status dg_batch_step(dg_batch* b, int32_t nsteps, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (b->dirty && (st = upload_tables(b, s))) return st;
   const bool use_graph = !(b->flags & DG_BATCH_NO_GRAPH);
-  if (use_graph && !b->graph[0] && (st = capture_graphs(b))) return st;
-  for (int32_t n = 0; n < nsteps; ++n) {
-    if (use_graph) {
-      cudaError_t err = cudaGraphLaunch(b->graph[b->cur], s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: graph launch");
-      b->launches += launches_per_step(b);
-    } else {
-      cudaError_t err = launch_step(b, b->cur, s);
-      if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: kernel launch");
+  const unsigned set = b->concurrent ? side_by_side(b) : 0;
+  if (set != 0 || !b->concurrent) {
+    if (use_graph && !b->graphs.count(set) && (st = capture_graphs(b, set))) return st;
+    for (int32_t n = 0; n < nsteps; ++n) {
+      const int src = b->cur ^ (n & 1);
+      if (use_graph) {
+        cudaError_t err = cudaGraphLaunch(b->graphs[set][src], s);
+        if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: graph launch");
+        b->launches += launches_per_step(b);
+      } else {
+        cudaError_t err = launch_step(b, src, s);
+        if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: kernel launch");
+      }
+      for (int g = 0; g < kOrders; ++g) b->steps[g] += ticked(b) >> g & 1;
     }
-    b->cur ^= 1;
-    ++b->steps;
   }
+  for (int g = 0; g < kOrders && nsteps > 0; ++g) {
+    if (!in_sequence(b, g)) continue;
+    const cudaError_t err = launch_order_steps(b, g, b->cur, nsteps, s);
+    if (err != cudaSuccess) return cuda_fail(err, "dg_batch_step: kernel launch");
+    b->steps[g] += nsteps;
+  }
+  b->cur ^= nsteps & 1;
   if (!(b->flags & DG_BATCH_NO_ADAPT) && !b->concurrent && nsteps > 0) {
     if (b->clock_pending && cudaEventQuery(b->clock_ev) == cudaSuccess) {
       b->clock_pending = false;
@@ -1013,20 +1104,24 @@ extern "C" dg_status dg_batch_tune(dg_batch* b, int32_t reps, void* stream) {
   //    keeps the split)
   if (err == cudaSuccess && !(b->flags & DG_BATCH_SPLIT)) {
     float conc_ms = 0.f;
-    err = launch_concurrent(b, b->cur, 1, 1, false, s);  // warm
+    const bool was = b->concurrent;
+    b->concurrent = true;  // which orders run alone in that mode
+    auto launch_orders = [&](int count) {
+      cudaError_t e = launch_concurrent(b, b->cur, 1, count, false, side_by_side(b), s);
+      for (int g = 0; g < kOrders && e == cudaSuccess; ++g)
+        if (in_sequence(b, g)) e = launch_chain(b, g, b->cur, 1, count, s);
+      return e;
+    };
+    err = launch_orders(1);  // warm
     if (err == cudaSuccess) err = cudaEventRecord(e0, s);
-    if (err == cudaSuccess) err = launch_concurrent(b, b->cur, 1, reps, false, s);
+    if (err == cudaSuccess) err = launch_orders(reps);
+    b->concurrent = was;
     if (err == cudaSuccess) err = cudaEventRecord(e1, s);
     if (err == cudaSuccess) err = cudaEventSynchronize(e1);
     if (err == cudaSuccess) err = cudaEventElapsedTime(&conc_ms, e0, e1);
     if (err == cudaSuccess) {
       const bool conc = conc_ms <= best_ms;
-      if (conc != b->concurrent) {
-        for (cudaGraphExec_t& g : b->graph) {
-          if (g) cudaGraphExecDestroy(g);
-          g = nullptr;
-        }
-      }
+      if (conc != b->concurrent) drop_graphs(b);
       b->concurrent = conc;
       b->tuned_split_ms = best_ms;
       b->tuned_concurrent_ms = conc_ms;

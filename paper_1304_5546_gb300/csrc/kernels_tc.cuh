@@ -450,8 +450,10 @@ __device__ __forceinline__ void media_flux(float nx, float ny, float cH, float c
 // both in the block is done once, by the lower-numbered element's task, for
 // both sides, with every flux operation explicitly rounded so that an
 // element's result does not depend on whether its neighbour shares its
-// block); otherwise each side's task computes its own face nodes.
-template <int N, int MODE, int PREC, bool MEDIA, bool TABLE, bool PAIRS = false, bool ALT = false>
+// block); otherwise each side's task computes its own face nodes.  CHAIN: the
+// launch may start before the launch before it ends (launch_chained).
+template <int N, int MODE, int PREC, bool MEDIA, bool TABLE, bool PAIRS = false, bool ALT = false,
+          bool CHAIN = !TABLE>
 __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const int first,
                                               const int G, unsigned char* smem) {
   using L = TcLayout<N, PREC, MEDIA, ALT>;
@@ -539,17 +541,17 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
     mbar_expect_tx(op_bar, L::NS * L::OB);
     tma_load_1d(smem + L::OFF_OP, p.tc_op, L::NS * L::OB, op_bar);
   };
-  // in a chain the tiles land while the launch before still runs; a batched
-  // launch is not chained, and its memory warp fetches them as it starts
-  // (here they measured 1.4 % slower there)
-  if (!TABLE && warp == L::IO_WARP && lane == 0 && !p.stall_gate) fetch_tiles();
+  // in a chain the tiles land while the launch before still runs; otherwise
+  // the memory warp fetches them as it starts (here they measured 1.4 %
+  // slower)
+  if (CHAIN && warp == L::IO_WARP && lane == 0 && !p.stall_gate) fetch_tiles();
   // flux threads: the face codes of the first block's tasks, straight from
   // global memory (no kernel of the chain writes them), so that its traces are
   // asked for at once, beside its stage's copies and not after them (a step
   // at N = 3, K = 1058 24.0 -> 22.9 us, at N = 6, K = 51,842 91.5 -> 89.8; in
   // the kernels of bf16x3 products and of batches, which have no registers
   // left for it, 135.6 -> 136.3 at N = 7, K = 49,928 and 0.15 % slower)
-  constexpr bool EARLY = !TABLE && PREC != kTcBf16x3;
+  constexpr bool EARLY = CHAIN && PREC != kTcBf16x3;
   int32_t code0[EARLY ? TPT : 1];
   if (EARLY && warp >= L::FLUX_WARP0 && warp < L::MMA_WARP && niter > 0) {
     int k0, nv;
@@ -563,7 +565,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
                      : -1;
     }
   }
-  if constexpr (!TABLE) {
+  if constexpr (CHAIN) {
     chain_wait();
     chain_trigger();
   }
@@ -650,7 +652,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
         ok = __shfl_sync(0xffffffffu, ok, 0);
       }
       if (ok) {
-        if ((TABLE || p.stall_gate) && lane == 0) fetch_tiles();
+        if ((!CHAIN || p.stall_gate) && lane == 0) fetch_tiles();
         for (; issued < niter && issued < S; ++issued) issue(issued);
       }
       for (int jj = 0; ok && jj < niter; ++jj) {
@@ -732,7 +734,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           }
         }
         if (ok) {
-          if (TABLE || p.stall_gate) fetch_tiles();
+          if (!CHAIN || p.stall_gate) fetch_tiles();
           for (; issued < niter && issued < S; ++issued) issue(issued);
         }
         // outputs of block jj leave by bulk stores, one bulk group per block
@@ -888,9 +890,9 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
             const int gP = (code >> 3) * Np + nbr[(code & 7) * Nfp + task_jj[u]];
             // a chained launch starts while the one before still writes these:
             // not the read-only path
-            trc[u][0] = TABLE ? __ldg(qin[0] + gP) : qin[0][gP];
-            trc[u][1] = TABLE ? __ldg(qin[1] + gP) : qin[1][gP];
-            trc[u][2] = TABLE ? __ldg(qin[2] + gP) : qin[2][gP];
+            trc[u][0] = CHAIN ? qin[0][gP] : __ldg(qin[0] + gP);
+            trc[u][1] = CHAIN ? qin[1][gP] : __ldg(qin[1] + gP);
+            trc[u][2] = CHAIN ? qin[2][gP] : __ldg(qin[2] + gP);
           }
         }
       }
@@ -1206,7 +1208,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           if (sid >= 0) {
             const double* m = p.src_meta + 4 * sid;
             const double t =
-                (static_cast<double>(__ldg(p.step_ctr) - __ldg(p.src_step + sid)) + p.c_stage) * m[0];
+                (static_cast<double>(__ldg(p.step_ctr) + p.step_off - __ldg(p.src_step + sid)) +
+                 p.c_stage) * m[0];
             const double aa = (t - m[1]) * m[2];
             samp = static_cast<float>(m[3] * (1.0 - 2.0 * aa * aa) * exp(-aa * aa));
             sw = p.src_w + sid * kSrcStride;
@@ -1417,13 +1420,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem[];
   if (static_cast<int>(blockIdx.x) >= __ldg(g.nblocks)) return;
   static_assert(TcLayout<N, kTcTf32x3, true, ALT>::THREADS == kTcThreads, "block size");
-  tc_stage_body<N, MODE, kTcTf32x3, true, true, false, ALT>(g, blockIdx.x, gridDim.x, smem);
+  tc_stage_body<N, MODE, kTcTf32x3, true, true, false, ALT, true>(g, blockIdx.x, gridDim.x, smem);
 }
 
 // ALT: the order's alternative block size (tc_tiles(N, prec, true)); the
 // block table must hold blocks of at most that many elements
 template <int N, int MODE, bool ALT>
-cudaError_t launch_batch_order(const StageArgs<float>& g, int grid, cudaStream_t stream) {
+cudaError_t launch_batch_order(const StageArgs<float>& g, int grid, bool chained,
+                               cudaStream_t stream) {
   if constexpr (ALT && !tc_has_alt(N, kTcTf32x3)) {
     return cudaErrorInvalidValue;
   } else {
@@ -1436,6 +1440,9 @@ cudaError_t launch_batch_order(const StageArgs<float>& g, int grid, cudaStream_t
     });
     if (err != cudaSuccess) return err;
     if (grid < 1) return cudaSuccess;
+    if (chained)
+      return launch_chained(dg_batch_order_kernel<N, MODE, ALT>, static_cast<unsigned>(grid),
+                            kTcThreads, L::SMEM_BYTES, stream, g);
     dg_batch_order_kernel<N, MODE, ALT><<<grid, kTcThreads, L::SMEM_BYTES, stream>>>(g);
     return cudaGetLastError();
   }

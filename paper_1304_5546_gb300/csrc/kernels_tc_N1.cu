@@ -7,10 +7,12 @@
 namespace dgw {
 template cudaError_t launch_stage_tc<1, kTcTf32x3>(const StageArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_stage_tc_media<1>(const StageArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_batch_order<1, kModeFirstStage>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_batch_order<1, kModeStage>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_batch_order<1, kModeFirstStage, true>(const StageArgs<float>&, int,
+template cudaError_t launch_batch_order<1, kModeFirstStage>(const StageArgs<float>&, int, bool,
+                                                      cudaStream_t);
+template cudaError_t launch_batch_order<1, kModeStage>(const StageArgs<float>&, int, bool,
+                                                      cudaStream_t);
+template cudaError_t launch_batch_order<1, kModeFirstStage, true>(const StageArgs<float>&, int, bool,
                                                                    cudaStream_t);
-template cudaError_t launch_batch_order<1, kModeStage, true>(const StageArgs<float>&, int,
+template cudaError_t launch_batch_order<1, kModeStage, true>(const StageArgs<float>&, int, bool,
                                                               cudaStream_t);
 }  // namespace dgw

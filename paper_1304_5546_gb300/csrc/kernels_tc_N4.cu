@@ -7,10 +7,12 @@
 namespace dgw {
 template cudaError_t launch_stage_tc<4, kTcTf32x3>(const StageArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_stage_tc_media<4>(const StageArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_batch_order<4, kModeFirstStage>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_batch_order<4, kModeStage>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_batch_order<4, kModeFirstStage, true>(const StageArgs<float>&, int,
+template cudaError_t launch_batch_order<4, kModeFirstStage>(const StageArgs<float>&, int, bool,
+                                                      cudaStream_t);
+template cudaError_t launch_batch_order<4, kModeStage>(const StageArgs<float>&, int, bool,
+                                                      cudaStream_t);
+template cudaError_t launch_batch_order<4, kModeFirstStage, true>(const StageArgs<float>&, int, bool,
                                                                    cudaStream_t);
-template cudaError_t launch_batch_order<4, kModeStage, true>(const StageArgs<float>&, int,
+template cudaError_t launch_batch_order<4, kModeStage, true>(const StageArgs<float>&, int, bool,
                                                               cudaStream_t);
 }  // namespace dgw

@@ -7,10 +7,12 @@
 namespace dgw {
 template cudaError_t launch_stage_tc<7, kTcTf32x3>(const StageArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_stage_tc_media<7>(const StageArgs<float>&, int, int, cudaStream_t);
-template cudaError_t launch_batch_order<7, kModeFirstStage>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_batch_order<7, kModeStage>(const StageArgs<float>&, int, cudaStream_t);
-template cudaError_t launch_batch_order<7, kModeFirstStage, true>(const StageArgs<float>&, int,
+template cudaError_t launch_batch_order<7, kModeFirstStage>(const StageArgs<float>&, int, bool,
+                                                      cudaStream_t);
+template cudaError_t launch_batch_order<7, kModeStage>(const StageArgs<float>&, int, bool,
+                                                      cudaStream_t);
+template cudaError_t launch_batch_order<7, kModeFirstStage, true>(const StageArgs<float>&, int, bool,
                                                                    cudaStream_t);
-template cudaError_t launch_batch_order<7, kModeStage, true>(const StageArgs<float>&, int,
+template cudaError_t launch_batch_order<7, kModeStage, true>(const StageArgs<float>&, int, bool,
                                                               cudaStream_t);
 }  // namespace dgw

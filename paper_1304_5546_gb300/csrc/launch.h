@@ -161,11 +161,12 @@ struct StageArgs {
   // projected point load times the problem's dt (src_w[index][kSrcStride])
   // and s the Ricker wavelet A (1 - 2 a^2) exp(-a^2), a = pi f (t - t0),
   // from src_meta[index] = {dt, t0, pi f, A}; the stage time is
-  // t = (step_ctr - src_step[index] + c_stage) dt.
+  // t = (step_ctr + step_off - src_step[index] + c_stage) dt.
   const float* src_w = nullptr;
   const double* src_meta = nullptr;
   const int* src_step = nullptr;
   const int* step_ctr = nullptr;
+  int step_off = 0;
   double c_stage = 0.0;
   // point source of a single operator (dg_operator_set_source): element
   // psrc_k (-1: none) gains psrc_amp * psrc_w[n] in its Ez residual, and b
@@ -344,7 +345,8 @@ cudaError_t launch_batch_tc(const BatchArgs& args, int grid, size_t smem, cudaSt
 // kernel of its own, `grid` CTAs (one per SM) over its block table
 // (g.blocks, g.nblocks); grid 0 only configures the kernel.
 template <int N, int MODE, bool ALT = false>
-cudaError_t launch_batch_order(const StageArgs<float>& g, int grid, cudaStream_t stream);
+cudaError_t launch_batch_order(const StageArgs<float>& g, int grid, bool chained,
+                               cudaStream_t stream);
 // shared memory and elements per block of order N's CTA in the batched launch
 // (alt: the alternative block size of the concurrent mode's kernels)
 size_t batch_tc_smem_bytes(int N, bool alt = false);
