@@ -862,6 +862,48 @@ dg_status copy_fields(dg_batch* b, int32_t slot, void* other, int64_t other_stri
 
 }  // namespace
 
+namespace {
+
+constexpr int kOutThreads = 256, kOutUnroll = 4;
+
+// The n values of fields f = blockIdx.y at q + f * fstride, to out + f * n in
+// host memory: thread 0 of a block on a 128-byte line of out, so that every
+// warp's store is a whole line on the way to the host.
+__global__ void __launch_bounds__(kOutThreads)
+    batch_out_kernel(const float* __restrict__ q, int64_t fstride, int64_t n, float* out) {
+  q += blockIdx.y * fstride;
+  out += blockIdx.y * n;
+  const int64_t head = static_cast<int64_t>((reinterpret_cast<uintptr_t>(out) / 4) % 32);
+  const int64_t j0 = static_cast<int64_t>(blockIdx.x) * (kOutThreads * kOutUnroll) - head + threadIdx.x;
+  float v[kOutUnroll];
+#pragma unroll
+  for (int u = 0; u < kOutUnroll; ++u) {
+    const int64_t j = j0 + u * kOutThreads;
+    v[u] = j >= 0 && j < n ? q[j] : 0.f;
+  }
+#pragma unroll
+  for (int u = 0; u < kOutUnroll; ++u) {
+    const int64_t j = j0 + u * kOutThreads;
+    if (j >= 0 && j < n) out[j] = v[u];
+  }
+}
+
+}  // namespace
+
+dg_status dgw::batch_fields_to_host(dg_batch* b, int32_t slot, float* out, cudaStream_t s) {
+  dg_status st = check_slot(b, slot, "dg_server");
+  if (st) return st;
+  const Problem& pr = b->probs[slot];
+  const Pool& p = b->pools[pr.N - 1];
+  const int64_t n = pr.K * p.Np, per = kOutThreads * kOutUnroll;
+  const dim3 grid(static_cast<unsigned>((n + 31 + per - 1) / per), 3);
+  batch_out_kernel<<<grid, kOutThreads, 0, s>>>(p.q[b->cur] + pr.off * p.Np, p.fstride, n, out);
+  const cudaError_t err = cudaGetLastError();
+  if (err != cudaSuccess) return cuda_fail(err, "dg_server: results");
+  ++b->launches;
+  return DG_OK;
+}
+
 extern "C" dg_status dg_batch_set_fields(dg_batch* b, int32_t slot, const void* src,
                                          int64_t src_stride, void* stream) {
   dgw::clear_error();

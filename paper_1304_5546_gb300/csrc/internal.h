@@ -175,6 +175,11 @@ void operator_records(const dg_op& op, std::vector<double>& rec, std::vector<int
 dg_status upload_operator(dg_op* op, const std::vector<double>& rec,
                           const std::vector<int32_t>& conn);
 
+// The fields of a batch's problem, asynchronously on stream s, to 3 K Np
+// contiguous floats at `out` (4-byte aligned) in memory that the device can
+// write.
+dg_status batch_fields_to_host(dg_batch* b, int32_t slot, float* out, cudaStream_t s);
+
 // One fused LSRK(5,4) stage (stage 0..4) of operator `op`: reads the fields
 // qin and the residual res, writes the updated fields to qout and the new
 // residual to res, asynchronously on stream s.
