@@ -56,14 +56,16 @@ def _ptr(a):
 def _stream_handle(stream):
     if stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the current stream's handle without a Stream object around it: 0.3 of
+        # 3.1 us of a call, and a small right-hand side is called in 7
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
-        return ctypes.c_void_p(stream)
-    return ctypes.c_void_p(stream.cuda_stream)
+        return stream
+    return stream.cuda_stream
 
 
 def _dptr(t):
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 # ------------------------------------------------------------------ mesh
