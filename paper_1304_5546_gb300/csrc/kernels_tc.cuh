@@ -83,6 +83,15 @@ struct TcLayout {
   static constexpr int ROWS = 3 * E;
   static constexpr int NPAD = tc_npad(N);
   static constexpr int IV = NPAD / 4;          // volume chunks of 4 nodes
+  // An element's row in the stage buffer is read and written 16 bytes at a
+  // time.  A warp's lanes hold consecutive elements, Np words apart: at N = 6
+  // and 7 (Np = 28 and 36) their 4-byte accesses meet 4-way bank conflicts,
+  // and 16-byte ones none.  GB300, us a step, 4 / 16 bytes: N = 7, BF16x3, K =
+  // 49,928 139.2 / 127.2; N = 6, K = 51,842 90.3 / 89.1 (TF32 products, K =
+  // 80,000 129.5 / 124.5); N = 7, K = 4232 43.8 / 43.1, K = 260,642 even; one
+  // TF32 or BF16 product at N = 7 175.8 / 176.8, 158.8 / 160.6: not there.  8
+  // bytes at N = 2 and 3 (2-way conflicts) measured 1 % slower.
+  static constexpr bool ROWS4 = N == 6 || (N == 7 && NS == 2);
   static constexpr int LCOLS = KP - 2 * NPAD;  // LIFT-part columns (zero beyond Nafp)
   // tensor memory: two accumulators, then XBUF operand buffers of NS parts.
   // Split variants (ACC_SPLIT): an accumulator has 2 NN columns, [0, NN)
@@ -158,6 +167,7 @@ struct TcLayout {
   // the flux warps wait for the next block's stage while on this one
   static_assert(S >= 3 && S <= 8, "stage ring / header layout");
   static_assert(SMEM_BYTES <= SMAX, "shared memory");
+  static_assert(!ROWS4 || (Np % 4 == 0 && NPAD == Np), "16-byte rows");
   static_assert(QB % 16 == 0 && GB % 16 == 0 && CB % 16 == 0 && OB % 16 == 0, "TMA chunks");
   static_assert(!LIFT_V4 || (FES % 4 == 0 && FES >= (Nafp + 3) / 4 * 4 && OFF_F % 16 == 0 &&
                              FB % 16 == 0),
@@ -203,6 +213,15 @@ struct RowShare {
   static constexpr int LLO = NR == 2 ? (ROLE == 0 ? L2 : 0) : (NR - 1 - ROLE) * LC / NR;
   static constexpr int LHI = NR == 2 ? (ROLE == 0 ? LC : L2) : (NR - ROLE) * LC / NR;
 };
+
+// Four consecutive values of an element's row in a stage buffer.
+__device__ __forceinline__ void row_load4(const float* p, float* v) {
+  const float4 x = *reinterpret_cast<const float4*>(p);
+  v[0] = x.x, v[1] = x.y, v[2] = x.z, v[3] = x.w;
+}
+__device__ __forceinline__ void row_store4(float* p, const float* v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
 
 // Four consecutive K columns (k0, a multiple of 4) of this thread's X row
 // into tensor memory at xh (and xl for the split variants), in the operand
@@ -325,6 +344,15 @@ __device__ __forceinline__ void build_x_vol(const float* qe, const float* lam, u
       const int m0 = 4 * (R::VLO + v);
       const float4 l2v = *reinterpret_cast<const float4*>(lam + m0);
       const float4 l3v = *reinterpret_cast<const float4*>(lam + NPAD + m0);
+      float uv[4], wv[4];  // u (and w) of the chunk's nodes
+      if constexpr (L::ROWS4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) uv[i] = a1, wv[i] = b1;
+        if (row_ok) {
+          row_load4(qe + fu + m0, uv);
+          if (rc == 2) row_load4(qe + E * Np + m0, wv);
+        }
+      }
 #pragma unroll
       for (int pp = 0; pp < 2; ++pp) {
         const int m = m0 + 2 * pp;
@@ -332,7 +360,8 @@ __device__ __forceinline__ void build_x_vol(const float* qe, const float* lam, u
         const f32x2 l3 = pp == 0 ? f32x2_pack(l3v.x, l3v.y) : f32x2_pack(l3v.z, l3v.w);
         const bool in0 = (L::ROW_LOADS_UNPRED || row_ok) && m < Np;
         const bool in1 = (L::ROW_LOADS_UNPRED || row_ok) && m + 1 < Np;
-        const f32x2 uq = f32x2_pack(in0 ? qe[fu + m] : a1, in1 ? qe[fu + m + 1] : a1);
+        const f32x2 uq = L::ROWS4 ? f32x2_pack(uv[2 * pp], uv[2 * pp + 1])
+                                  : f32x2_pack(in0 ? qe[fu + m] : a1, in1 ? qe[fu + m + 1] : a1);
         f32x2 ud = f32x2_sub(uq, f32x2_dup(a1));
         if constexpr (L::DEFL_FMA) {
           ud = f32x2_fma(f32x2_dup(a1 - a2), l2, ud);
@@ -343,7 +372,9 @@ __device__ __forceinline__ void build_x_vol(const float* qe, const float* lam, u
         f32x2 pr = f32x2_mul(f32x2_dup(rc == 1 ? rx : -ry), ud);
         f32x2 ps = f32x2_mul(f32x2_dup(rc == 1 ? sx : -sy), ud);
         if (rc == 2) {
-          const f32x2 wq = f32x2_pack(in0 ? qe[E * Np + m] : b1, in1 ? qe[E * Np + m + 1] : b1);
+          const f32x2 wq =
+              L::ROWS4 ? f32x2_pack(wv[2 * pp], wv[2 * pp + 1])
+                       : f32x2_pack(in0 ? qe[E * Np + m] : b1, in1 ? qe[E * Np + m + 1] : b1);
           f32x2 wd = f32x2_sub(wq, f32x2_dup(b1));
           if constexpr (L::DEFL_FMA) {
             wd = f32x2_fma(f32x2_dup(b1 - b2), l2, wd);
@@ -1221,17 +1252,41 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           float* rq = sq + c * E * Np + e * Np;
           float* rr = sres + c * E * Np + e * Np;
           const f32x2 a2 = f32x2_dup(p.a), b2 = f32x2_dup(p.b), dt2 = f32x2_dup(drow);
+          if constexpr (L::ROWS4) {
 #pragma unroll
-          for (int n = 0; n + 1 < Np; n += 2) {
-            if (MODE == kModeRhs) {
-              rq[n] = MEDIA ? srow * acc[n] : acc[n];
-              rq[n + 1] = MEDIA ? srow * acc[n + 1] : acc[n + 1];
-            } else {
-              f32x2 rn = f32x2_mul(dt2, f32x2_pack(acc[n], acc[n + 1]));
-              if (MODE == kModeStage) rn = f32x2_fma(a2, f32x2_pack(rr[n], rr[n + 1]), rn);
-              const f32x2 qn = f32x2_fma(b2, rn, f32x2_pack(rq[n], rq[n + 1]));
-              f32x2_unpack(qn, rq[n], rq[n + 1]);
-              f32x2_unpack(rn, rr[n], rr[n + 1]);
+            for (int n = 0; n < Np; n += 4) {
+              float vq[4], vr[4];
+              if (MODE == kModeRhs) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) vq[i] = MEDIA ? srow * acc[n + i] : acc[n + i];
+              } else {
+                row_load4(rq + n, vq);
+                if (MODE == kModeStage) row_load4(rr + n, vr);
+#pragma unroll
+                for (int i = 0; i < 4; i += 2) {
+                  f32x2 rn = f32x2_mul(dt2, f32x2_pack(acc[n + i], acc[n + i + 1]));
+                  if (MODE == kModeStage) rn = f32x2_fma(a2, f32x2_pack(vr[i], vr[i + 1]), rn);
+                  const f32x2 qn = f32x2_fma(b2, rn, f32x2_pack(vq[i], vq[i + 1]));
+                  f32x2_unpack(qn, vq[i], vq[i + 1]);
+                  f32x2_unpack(rn, vr[i], vr[i + 1]);
+                }
+                row_store4(rr + n, vr);
+              }
+              row_store4(rq + n, vq);
+            }
+          } else {
+#pragma unroll
+            for (int n = 0; n + 1 < Np; n += 2) {
+              if (MODE == kModeRhs) {
+                rq[n] = MEDIA ? srow * acc[n] : acc[n];
+                rq[n + 1] = MEDIA ? srow * acc[n + 1] : acc[n + 1];
+              } else {
+                f32x2 rn = f32x2_mul(dt2, f32x2_pack(acc[n], acc[n + 1]));
+                if (MODE == kModeStage) rn = f32x2_fma(a2, f32x2_pack(rr[n], rr[n + 1]), rn);
+                const f32x2 qn = f32x2_fma(b2, rn, f32x2_pack(rq[n], rq[n + 1]));
+                f32x2_unpack(qn, rq[n], rq[n + 1]);
+                f32x2_unpack(rn, rr[n], rr[n + 1]);
+              }
             }
           }
           if (Np & 1) {
