@@ -118,6 +118,14 @@ struct TcLayout {
   // at N >= 5 (2-9 % faster there on GB300), by lane 0 alone at N <= 4
   // (where several issuing lanes measured 2-6 % slower)
   static constexpr bool IO_LANES = N >= 5;
+  // The memory warp refills a stage as soon as its own stores have read it,
+  // at N = 7 with split products, where four stages are all that fit and the
+  // flux warps wait 2300 of a block's 5000 clocks for the next one: us a step,
+  // K = 260,642 554.8 -> 543.0, K = 555,458 1167 -> 1141, BF16x3, K = 49,928
+  // 125.8 -> 124.0.  Elsewhere it refills the stage of the block before, and
+  // never waits for the stores it has just issued (N = 6, K = 320,000 447
+  // against 454; N = 7, one TF32 product 172 against 174.7; N <= 5 even).
+  static constexpr bool REFILL_OWN = N == 7 && NS == 2;
   // widest tcgen05.st of an operand-row run (columns): 8 (1-4 % faster than
   // 4 at every order on GB300), 16 at N = 7 (where it measured faster
   // still; at N = 6 it was slower than 8)
@@ -709,7 +717,15 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
           }
         }
         bulk_commit();
-        if (jj >= 1 && issued < niter) {  // issued == jj - 1 + S: the stage of block jj - 1
+        if constexpr (L::REFILL_OWN) {
+          if (issued < niter) {  // issued == jj + S: the stage of this block
+            bulk_wait_read_all();
+            __syncwarp();
+            fence_proxy_async();
+            issue(issued);
+            ++issued;
+          }
+        } else if (jj >= 1 && issued < niter) {  // jj - 1 + S: the stage of block jj - 1
           bulk_wait_read_but_last();
           __syncwarp();
           fence_proxy_async();
