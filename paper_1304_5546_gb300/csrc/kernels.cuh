@@ -211,12 +211,15 @@ __global__ void __launch_bounds__(Layout<N, MEDIA, E_>::THREADS)
 
   // face codes of the first block's tasks, straight from global memory (no
   // kernel of the chain writes them): its traces are asked for beside its
-  // stage's copies, not after them
+  // stage's copies, not after them (a step at N = 4, K = 45,000 100.5 -> 97.6
+  // us; at N = 3 without a permittivity the blocks of 32 elements lose by it:
+  // K = 39,762 50.1 -> 55.6, K = 249,218 247 -> 277)
+  constexpr bool EARLY = E < simt_block_elems(N) || N != 3 || MEDIA;
   int32_t code0[TPT];
 #pragma unroll
   for (int u = 0; u < TPT; ++u) {
     const int k = first * E + task_e[u];
-    code0[u] = niter > 0 && task_e[u] < E && k < K
+    code0[u] = EARLY && niter > 0 && task_e[u] < E && k < K
                    ? __ldg(p.conn + static_cast<int64_t>(k) * 3 + task_f[u])
                    : -1;
   }
@@ -239,7 +242,7 @@ __global__ void __launch_bounds__(Layout<N, MEDIA, E_>::THREADS)
       trc[u][0] = trc[u][1] = trc[u][2] = 0.f;
       const int ee = task_e[u];
       if (ee < E && k0 + ee < K) {
-        const int32_t code = at_start ? code0[u] : sc[ee * 3 + task_f[u]];
+        const int32_t code = EARLY && at_start ? code0[u] : sc[ee * 3 + task_f[u]];
 #ifdef DGW_DEVICE_CHECKS
         if (!nbr_code_ok(code, p.fstride, Np)) {
           atomicOr(p.status, kStatusIndex);
@@ -257,7 +260,10 @@ __global__ void __launch_bounds__(Layout<N, MEDIA, E_>::THREADS)
   };
 
   bool ok = true;
-  if (niter > 0) gather(0, true);
+  if (niter > 0) {
+    if (!EARLY) ok = mbar_wait_bounded(&bars[0], 0, kWaitLimitNs);
+    if (ok) gather(0, true);
+  }
 
   int it = 0;
   for (; it < niter; ++it) {
