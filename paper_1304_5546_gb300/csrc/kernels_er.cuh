@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(ErLayout<N, MEDIA>::THREADS, 1)
       float* sq = q_stage(j);
       float* sr = r_stage(j);
       const int se = p.psrc_k - k0;
-      if (p.psrc_k >= 0 && se >= 0 && se < nv) {  // the operator's point source
+      if (static_cast<unsigned>(se) < static_cast<unsigned>(nv)) {  // the operator's point source
         float* y = sq + 2 * E * Np + se * Np;
         float* r = sr + 2 * E * Np + se * Np;
         if (nv != E) {
@@ -291,16 +291,7 @@ __global__ void __launch_bounds__(ErLayout<N, MEDIA>::THREADS, 1)
           y = (MODE == kModeRhs ? p.rhs : p.qout) + g;
           r = p.res + g;
         }
-        for (int n = lane; n < Np; n += 32) {
-          const float wn = __ldg(p.psrc_w + n);
-          if (MODE == kModeRhs) {
-            y[n] = __fmaf_rn(p.psrc_amp, wn, y[n]);
-          } else {
-            const float v = __fmul_rn(p.psrc_amp, wn);
-            r[n] = __fadd_rn(r[n], v);
-            y[n] = __fmaf_rn(p.b, v, y[n]);
-          }
-        }
+        point_source_call<Np, MODE>(y, r, p.psrc_w, p.psrc_amp, p.b, lane, 32);
         fence_proxy_async();
       }
       __syncwarp();

@@ -482,6 +482,34 @@ __device__ __forceinline__ void media_flux(float nx, float ny, float cH, float c
   fz = f;
 }
 
+// A point source on one element's Ez row: y (values, or right-hand side) and r
+// (residual) gain it at nodes l0, l0 + step, ...
+template <int Np, int MODE>
+__device__ __forceinline__ void point_source_row(float* y, float* r, const float* weights,
+                                                 float amp, float b, int l0, int step) {
+#pragma unroll 1
+  for (int n = l0; n < Np; n += step) {
+    const float w = __ldg(weights + n);
+    if (MODE == kModeRhs) {
+      y[n] = __fmaf_rn(amp, w, y[n]);
+    } else {
+      const float v = __fmul_rn(amp, w);
+      r[n] = __fadd_rn(r[n], v);
+      y[n] = __fmaf_rn(b, v, y[n]);
+    }
+  }
+}
+// The same as a call: inlined, the lines that one block of a launch runs slow
+// the memory warp down in all of them.  GB300, us a step, inlined / called: N =
+// 7, K = 249,218 533.9 / 519.1; N = 6, BF16x3, K = 320,000 465.1 / 457.1; N =
+// 3, BF16x3, K = 897,800 615.5 / 594.2; even at N = 4 and 5; N = 1, BF16x3, K =
+// 3.0M 1282 / 1295 and N = 2 173.4 / 174.0: inlined at N <= 2.
+template <int Np, int MODE>
+__device__ __noinline__ void point_source_call(float* y, float* r, const float* weights, float amp,
+                                               float b, int l0, int step) {
+  point_source_row<Np, MODE>(y, r, weights, amp, b, l0, step);
+}
+
 // One CTA's share of a stage launch: the blocks first, first + G, ... of
 // the launch (TABLE: from the block table p.blocks; else contiguous blocks of
 // E elements over [0, K)).  smem: the CTA's dynamic shared memory (1024-byte
@@ -588,9 +616,9 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
   // global memory (no kernel of the chain writes them), so that its traces are
   // asked for at once, beside its stage's copies and not after them (a step
   // at N = 3, K = 1058 24.0 -> 22.9 us, at N = 6, K = 51,842 91.5 -> 89.8; in
-  // the kernels of bf16x3 products and of batches, which have no registers
-  // left for it, 135.6 -> 136.3 at N = 7, K = 49,928 and 0.15 % slower)
-  constexpr bool EARLY = CHAIN && PREC != kTcBf16x3;
+  // the kernels of bf16x3 products, 135.6 -> 136.3 at N = 7, K = 49,928, and
+  // of single TF32 products at N = 7, K = 249,218 505 -> 520, it costs more)
+  constexpr bool EARLY = CHAIN && PREC != kTcBf16x3 && !(N == 7 && PREC == kTcTf32);
   int32_t code0[EARLY ? TPT : 1];
   if (EARLY && warp >= L::FLUX_WARP0 && warp < L::MMA_WARP && niter > 0) {
     int k0, nv;
@@ -622,24 +650,15 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs<float>& p, const i
   auto add_source = [&](int k0, int nv, float* sq, int l0, int step) {
     if constexpr (!TABLE) {
       const int e = p.psrc_k - k0;
-      if (p.psrc_k < 0 || e < 0 || e >= nv) return;
-      float* y = sq + 2 * E * Np + e * Np;  // Ez values (or right-hand side)
-      float* r = y + 3 * E * Np;
-      if (nv != E) {
-        const int64_t g = 2 * fs + static_cast<int64_t>(p.psrc_k) * Np;
-        y = (MODE == kModeRhs ? p.rhs : p.qout) + g;
-        r = p.res + g;
-      }
-      for (int n = l0; n < Np; n += step) {
-        const float w = __ldg(p.psrc_w + n);
-        if (MODE == kModeRhs) {
-          y[n] = __fmaf_rn(p.psrc_amp, w, y[n]);
-        } else {
-          const float v = __fmul_rn(p.psrc_amp, w);
-          r[n] = __fadd_rn(r[n], v);
-          y[n] = __fmaf_rn(p.b, v, y[n]);
-        }
-      }
+      if (static_cast<unsigned>(e) >= static_cast<unsigned>(nv)) return;
+      const int o = 2 * E * Np + e * Np;  // Ez values (or right-hand side)
+      const int64_t g = 2 * fs + static_cast<int64_t>(p.psrc_k) * Np;
+      float* y = nv == E ? sq + o : (MODE == kModeRhs ? p.rhs : p.qout) + g;
+      float* r = nv == E ? sq + 3 * E * Np + o : p.res + g;
+      if constexpr (N <= 2)
+        point_source_row<Np, MODE>(y, r, p.psrc_w, p.psrc_amp, p.b, l0, step);
+      else
+        point_source_call<Np, MODE>(y, r, p.psrc_w, p.psrc_amp, p.b, l0, step);
       fence_proxy_async();
     }
   };
