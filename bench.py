@@ -425,7 +425,8 @@ def run_ours(args):
             "frac": achieved / peaks["hbm_gbs"],
             "traffic": traffic,
             "peak_kind": peak_kind,
-            "kernel": {"tensor cores": "dg_stage_tc_kernel", "cuda cores": "dg_stage_kernel",
+            "kernel": {"tensor cores": "dg_stage_er_kernel" if s.kernel()[1] == 128
+                       else "dg_stage_tc_kernel", "cuda cores": "dg_stage_kernel",
                        "element threads": "dg_stage_ept_kernel"}[kernel_kind]
                       + " (fused RHS + LSRK stage)",
             "bytes_per_element_step": step_bytes_per_element(N),
