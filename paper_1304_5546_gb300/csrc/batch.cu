@@ -44,7 +44,7 @@ using dgw::fail;
 namespace {
 
 constexpr int kOrders = DG_N_MAX;
-constexpr size_t kMaxGraphs = 8;  // sets of orders whose step graphs are kept
+constexpr size_t kMaxGraphs = 32;  // sets of orders whose step graphs are kept
 constexpr int kPadElems = 8;  // pool tail read by the last block's 16-byte rounding
 
 dg_status cuda_fail(cudaError_t err, const char* where) {
@@ -408,12 +408,18 @@ void plan_sequence(dg_batch* b) {
 
 bool in_sequence(const dg_batch* b, int g) { return b->concurrent && b->alone[g]; }
 
-// The other orders with blocks, as a bit mask.
+// The other orders, as a bit mask; 0 if none of them has blocks.  Orders
+// without blocks are among them (their CTAs return at once), so that the set,
+// and with it the step graph, does not change with every join and leave.
 unsigned side_by_side(const dg_batch* b) {
   unsigned mask = 0;
-  for (int g = 0; g < kOrders; ++g)
-    if (b->nblk[g] > 0 && !in_sequence(b, g)) mask |= 1u << g;
-  return mask;
+  bool any = false;
+  for (int g = 0; g < kOrders; ++g) {
+    if (b->pools[g].cap == 0 || in_sequence(b, g)) continue;
+    mask |= 1u << g;
+    any = any || b->nblk[g] > 0;
+  }
+  return any ? mask : 0;
 }
 
 // The orders whose step counters launch_step advances.
