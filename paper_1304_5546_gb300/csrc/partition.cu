@@ -292,10 +292,12 @@ dg_status build_device(dg_partition& pt) {
     s->ref = op.ref;
     s->alpha = op.alpha;
     s->face_pairs = op.face_pairs;
+    // the operator's kernel, whatever the part's size: results equal bit for bit
     s->use_tc = op.use_tc;
     s->use_ept = op.use_ept;
     s->tc_prec = op.tc_prec;
-    s->use_er = op.use_er;  // the same kernel whatever the part's size: results equal bit for bit
+    s->tc_alt = op.tc_alt;  // decides between the element-row kernel and the other one too
+    s->use_er = op.use_er;
     s->er_off = op.er_off;
     s->small = op.small;
     s->small_off = op.small_off;

@@ -1,0 +1,52 @@
+"""GPU: the kernel and block size of an FP32 operator as its caller sees and
+sets them (dg_operator_kernel, dg_operator_set_block_elems, dg_operator_tune),
+and partitions of an operator on a size that was set.
+"""
+import numpy as np
+import pytest
+
+from synth import jittered_delaunay_mesh, random_permittivity
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need CUDA"
+    from paper_1304_5546_gb300 import build as B
+    B.build()
+    import paper_1304_5546_gb300 as P
+    return P
+
+
+def _mesh(K):
+    n = int(np.ceil(np.sqrt(K / 2)))
+    VX, VY, E = jittered_delaunay_mesh(n, seed=5)
+    used, E = np.unique(E[:K], return_inverse=True)
+    return VX[used], VY[used], E.reshape(-1, 3).astype(np.int32)
+
+
+# an operator of the element-row kernel on the other tensor-core kernel: in
+# its default and in its alternative size, whose parts must run that one too
+@pytest.mark.parametrize("N,elems,media", [(3, 40, False), (3, 80, False), (4, 80, False),
+                                           (4, 40, True), (4, 80, True), (5, 40, False)])
+def test_partition_runs_the_kernel_that_was_set(P, N, elems, media):
+    import torch
+    mesh = _mesh(40000)
+    eps = random_permittivity(40000, seed=3) if media else None
+    s = P.Solver(*mesh, N=N, eps=eps)
+    assert s.kernel() == ("tensor cores", 128)
+    P.dg_operator_set_block_elems(s.op, elems)
+    assert s.kernel() == ("tensor cores", elems)
+    q0 = s.from_numpy(np.random.default_rng(1).uniform(-1, 1, (3, s.K, s.Np)))
+    res, want, got, dt = s.new_fields(), q0.clone(), s.new_fields(), s.cfl_dt()
+    s.step(want, res, dt, 2)
+    part = P.Partition(s, 3)
+    part.set_fields(q0)
+    part.step(dt, 2)
+    part.get_fields(got)
+    part.sync_check()
+    P.dg_sync_check(s.op)
+    assert torch.equal(s.view(got), s.view(want))
+    s.close()
