@@ -218,9 +218,10 @@ std::vector<unsigned char> er_operator_tiles(const dgw::RefElement& R, bool medi
   return bytes;
 }
 
-// Dr, Ds and LIFT in fixed point for the FP64 kernel (f64_table_pairs,
-// launch.h): v = (hi 2^28 + lo) 2^scale, at most 2^55 in size, with a scale
-// per node for its rows of Dr and Ds and one for its row of LIFT.
+// Dr, Ds and LIFT in fixed point for the FP64 kernel (f64_table_ints,
+// launch.h): v = (x 2^56 + y 2^28 + z) 2^scale, below 2^83 in size, each limb at
+// most 2^27, with a scale per node for its rows of Dr and Ds and one for its row
+// of LIFT.  Exact for entries down to 2^-30 of their row's largest.
 std::vector<unsigned char> f64_operator_table(const dgw::RefElement& R) {
   const int N = R.N, Np = R.Np, Nafp = R.Nafp;
   std::vector<int> sd(Np), sl(Np);
@@ -229,22 +230,37 @@ std::vector<unsigned char> f64_operator_table(const dgw::RefElement& R) {
     for (int m = 0; m < Np; ++m)
       d = std::max({d, std::fabs(R.Dr[n * Np + m]), std::fabs(R.Ds[n * Np + m])});
     for (int j = 0; j < Nafp; ++j) l = std::max(l, std::fabs(R.LIFT[n * Nafp + j]));
-    sd[n] = std::ilogb(d) + 1 - 55;
-    sl[n] = std::ilogb(l) + 1 - 55;
+    sd[n] = std::ilogb(d) + 1 - 83;
+    sl[n] = std::ilogb(l) + 1 - 83;
   }
-  std::vector<int32_t> out;
-  auto put = [&](double v, int scale) {
-    const int64_t n = std::llround(std::ldexp(v, -scale));
-    const int64_t lo = ((n + (1 << 27)) & ((1 << 28) - 1)) - (1 << 27);
-    out.push_back(static_cast<int32_t>((n - lo) >> 28));
-    out.push_back(static_cast<int32_t>(lo));
+  std::vector<int32_t> out(dgw::f64_table_ints(N), 0);
+  auto limbs = [](double v, int scale, int32_t* l) {
+    double x = std::ldexp(v, -scale);  // what is taken off it leaves it exact
+    for (int i = 0; i < 3; ++i) {
+      const double t = std::nearbyint(std::ldexp(x, 28 * (i - 2)));
+      x -= std::ldexp(t, 28 * (2 - i));
+      l[i] = static_cast<int32_t>(t);
+    }
   };
-  for (const std::vector<double>* D : {&R.Dr, &R.Ds})
-    for (int c = 0; c < Np - 3; ++c)
-      for (int n = 0; n < Np; ++n) put((*D)[n * Np + (c < N - 1 ? c + 1 : c + 2)], sd[n]);
+  const size_t nv = static_cast<size_t>(Np - 3) * Np, nl = static_cast<size_t>(Nafp) * Np;
+  for (int c = 0; c < Np - 3; ++c)
+    for (int n = 0; n < Np; ++n) {
+      const int m = n * Np + (c < N - 1 ? c + 1 : c + 2);
+      const size_t at = static_cast<size_t>(c) * Np + n;
+      int32_t r[3], s[3];
+      limbs(R.Dr[m], sd[n], r);
+      limbs(R.Ds[m], sd[n], s);
+      out[4 * at] = r[0], out[4 * at + 1] = r[1], out[4 * at + 2] = s[0], out[4 * at + 3] = s[1];
+      out[4 * nv + 2 * at] = r[2], out[4 * nv + 2 * at + 1] = s[2];
+    }
   for (int j = 0; j < Nafp; ++j)
-    for (int n = 0; n < Np; ++n) put(R.LIFT[n * Nafp + j], sl[n]);
-  out.resize(2 * static_cast<size_t>(dgw::f64_table_pairs(N)), 0);
+    for (int n = 0; n < Np; ++n) {
+      const size_t at = static_cast<size_t>(j) * Np + n;
+      int32_t l[3];
+      limbs(R.LIFT[n * Nafp + j], sl[n], l);
+      out[6 * nv + 2 * at] = l[0], out[6 * nv + 2 * at + 1] = l[1];
+      out[6 * nv + 2 * nl + at] = l[2];
+    }
   for (int n = 0; n < Np; ++n) {
     out.push_back(sd[n]);
     out.push_back(sl[n]);

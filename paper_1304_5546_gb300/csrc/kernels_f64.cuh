@@ -14,12 +14,23 @@
 // * Products in fixed point.  The operand vectors of an element (deflated
 //   Ez; A = rx Hy - ry Hx and B = sx Hy - sy Hx, deflated; the face fluxes)
 //   are scaled by a power of two taken from the vector's largest entry and
-//   rounded to 56-bit integers v = hi 2^28 + lo (28-bit signed limbs), and so,
-//   on the host, are the rows of Dr, Ds and LIFT.  A term is four 32 x 32 ->
-//   64 bit multiply-adds into the sums of hi hi, of hi lo + lo hi and of lo
-//   lo, which are exact (|hi| <= 2^27, at most 66 terms).  Rounding an entry
-//   to 2^-56 of its vector's (its row's) largest and one final rounding
-//   replace the roundings of up to 60 FP64 multiply-adds.
+//   taken as 84-bit integers hi 2^56 + mid 2^28 + lo (28-bit signed limbs),
+//   and so, on the host, are the rows of Dr, Ds and LIFT.  An entry keeps its
+//   53 bits down to 2^-31 of its vector's (its row's) largest.  A term is six
+//   32 x 32 -> 64 bit multiply-adds into the sums of hi hi, of hi mid + mid hi
+//   and of hi lo + mid mid + lo hi, which are exact (operand limbs below 2^28,
+//   table limbs at most 2^27, at most 66 terms); what is left out is 2^-82 of
+//   the largest product.  One final rounding replaces the roundings of up to
+//   60 FP64 multiply-adds, and a component that only small entries reach is
+//   as precise as they are: rows of Dr at N = 3, 5, 7 times vectors with
+//   entries over nine decades, largest relative error of a component, FMAs /
+//   two limbs (56 bits) / three: 2.6e-14 / 1.3e-8 / 1.1e-16 (over twelve, where
+//   entries lose bits, 1.7e-14 / 1.2e-5 / 2.9e-14).  With two limbs an element
+//   beside one 1e8 times larger, on axis-aligned faces, had components off by
+//   1e7 times 2^-53 of their own terms' sizes (now 32 at most).  They are
+//   faster: GB300, us a step, two / three limbs: N = 1, K = 180,000 302 / 320; 2,
+//   80,000 324 / 354; 3, 45,000 305 / 337; 4, 45,000 397 / 439; 5, 101,250 1270 /
+//   1453; 6, 20,000 363 / 472; 7, 20,000 534 / 695; N = 4, K = 128 32.5 / 37.4.
 // * An operand vector that fixed point cannot hold -- largest entry
 //   infinite, NaN, or outside 2^-890 .. 2^870 -- keeps its FP64 values in the
 //   same slots, and its element takes the products in FP64.
@@ -54,29 +65,30 @@ namespace dgw {
 // Resident CTAs the register allocation aims at, and product columns per
 // unrolled step.  More CTAs let one's products run beside another's FP64
 // phases, until the registers spill (us a step on the meshes of
-// f64_max_elems' table, CTAs aimed at: N = 1 2 / 3 / 4 358 / 309 / 313, N = 2
-// 4 / 6 383 / 326, N = 3 3 / 4 / 5 348 / 312 / 320, N = 5 2 / 3 / 4 / 5 1506 /
-// 1395 / 1331 / 1364, N = 7 2 / 3 / 4 601 / 560 / 575; three columns a step
-// instead of two: N = 5 1292, N = 6 371 against 378, N = 7 605 against 575).
-__host__ __device__ constexpr int f64_ctas(int N) { return N == 1 || N == 7 ? 3 : N == 2 ? 6 : 4; }
-__host__ __device__ constexpr int f64_unroll(int N) { return N == 7 ? 2 : 3; }
+// f64_max_elems' table, CTAs aimed at: N = 1 2 / 3 / 4 / 5 377 / 332 / 320 /
+// 337, N = 2 2 / 4 / 5 / 6 405 / 405 / 358 / 354, N = 3 2 / 3 / 4 / 5 432 / 379 /
+// 337 / 348, N = 5 1713 / 1664 / 1510 / 1651, N = 7 720 / 760 / 717 / 726; three
+// / four / six columns a step: N = 3 337 / 345 / 344, N = 4 439 / 439 / 465, N =
+// 5 1510 / 1453 / 1565, N = 6 484 / 472 / 468, N = 7 717 / 695 / 695).
+__host__ __device__ constexpr int f64_ctas(int N) { return N == 2 ? 6 : 4; }
+__host__ __device__ constexpr int f64_unroll(int N) { return N <= 4 ? 3 : 4; }
 
 template <int N, bool MEDIA>
 struct F64Layout {
   static constexpr int Np = Order<N>::Np, Nfp = Order<N>::Nfp, Nafp = Order<N>::Nafp;
   static constexpr int GEO = MEDIA ? kGeoMedia : kGeo;
   static constexpr int NI = Np - 3;  // nodes that are not vertices
-  static constexpr int TABLE = f64_table_pairs(N);            // limb pairs
+  static constexpr int TABLE = f64_table_ints(N);
   static constexpr int TPT = (Nafp + Np - 1) / Np;            // flux tasks per thread
   // shared memory of a block of E elements: table, then per stage buffer
   // q[3], res[3], geometry, codes; then operands, differences, linear terms,
-  // maxima
+  // maxima, the rest of the operands (two: with the second flux scalar's)
   __host__ __device__ static constexpr int stage_bytes(int E) {
-    return E * (6 * Np * 8 + GEO * 8) + (E * 12 + 7) / 8 * 8;
+    return (E * (6 * Np * 8 + GEO * 8 + 12) + 15) / 16 * 16;
   }
-  static constexpr int OPS = 3 * NI + 2 * Nafp;  // operand slots (8 bytes) of an element
-  __host__ __device__ static constexpr int smem_bytes(int E) {
-    return 8 * TABLE + 2 * stage_bytes(E) + E * (OPS * 8 + 6 * 8 + 3 * 8 + 2 * 4 * 4);
+  __host__ __device__ static constexpr int smem_bytes(int E, bool two) {
+    return 4 * TABLE + 2 * stage_bytes(E) +
+           E * (NI * 36 + (two ? 2 : 1) * Nafp * 16 + 6 * 8 + 3 * 8 + 2 * 4 * 4);
   }
 };
 
@@ -100,27 +112,40 @@ __device__ __forceinline__ bool f64_fixed(int size) {
   return size == 0 || (e >= 128 && e <= 1900);
 }
 
-// v / 2^(ex - 1077) rounded to an integer of at most 2^55, ex the biased
-// exponent of its vector's largest entry, as limbs x 2^28 + y, |y| <= 2^27
-__device__ __forceinline__ int2 f64_limbs(double v, int ex) {
+// A fixed-point number x 2^56 + y 2^28 + z.
+struct F64Limbs {
+  int x, y, z;
+};
+
+// v 2^(1106 - ex) cut to an integer below 2^84 in size, ex the biased exponent
+// of its vector's largest entry (exact if v's is at least ex - 31)
+__device__ __forceinline__ F64Limbs f64_limbs(double v, int ex) {
   const long long b = __double_as_longlong(v);
   const int e = static_cast<int>((b >> 52) & 0x7ff);
-  long long m = (b & 0xfffffffffffffll) | (e ? 1ll << 52 : 0);
+  const unsigned long long m =
+      (static_cast<unsigned long long>(b) << 11) | (e ? 1ull << 63 : 0);
   const int sh = ex - (e ? e : 1);
-  m = (((m << 3) >> (sh < 63 ? sh : 63)) + 1) >> 1;
-  if (b < 0) m = -m;
-  const int lo = static_cast<int>(static_cast<unsigned>(m) << 4) >> 4;
-  return make_int2(static_cast<int>((m - lo) >> 28), lo);
+  // the integer's upper 64 bits and the 20 below them
+  const unsigned long long top = sh < 64 ? m >> sh : 0;
+  const unsigned long long below =
+      sh == 0 ? 0 : sh < 64 ? m << (64 - sh) : sh < 128 ? m >> (sh - 64) : 0;
+  const int x = static_cast<int>(top >> 36);
+  const int y = static_cast<int>((top >> 8) & 0xfffffff);
+  const int z = static_cast<int>(((top & 0xff) << 20) | (below >> 44));
+  return b < 0 ? F64Limbs{-x, -y, -z} : F64Limbs{x, y, z};
 }
 
-// A sum of fixed-point products, hh 2^56 + hl 2^28 + ll (|hh| < 2^61)
+// A sum of fixed-point products, without their parts below 2^56: (hh 2^56 +
+// hl 2^28 + ll) 2^56
 struct F64Sum {
   long long hh = 0, hl = 0, ll = 0;
-  __device__ __forceinline__ void term(int2 a, int2 b) {
+  __device__ __forceinline__ void term(const F64Limbs& a, const F64Limbs& b) {
     hh += static_cast<long long>(a.x) * b.x;
     hl += static_cast<long long>(a.x) * b.y;
     hl += static_cast<long long>(a.y) * b.x;
+    ll += static_cast<long long>(a.x) * b.z;
     ll += static_cast<long long>(a.y) * b.y;
+    ll += static_cast<long long>(a.z) * b.x;
   }
   __device__ __forceinline__ void add(const F64Sum& o) {
     hh += o.hh;
@@ -129,16 +154,30 @@ struct F64Sum {
   }
 };
 
-// The FP64 value of a sum times its operands' powers of two, 2^(ex - 1077)
+// The FP64 value of a sum times its operands' powers of two, 2^(ex - 1106)
 // and 2^scale; k = ex + scale
 __device__ __forceinline__ double f64_value(const F64Sum& s, int k) {
-  const long long r = (s.hh << 2) + ((s.hl + (s.ll >> 28)) >> 26);
-  if (r == 0) return 0.0;
-  unsigned long long a = r < 0 ? -static_cast<unsigned long long>(r) : r;
-  const int lz = __clzll(a);
-  a = ((a << lz) + (1ull << 10)) >> 11;  // 53 bits, or 2^53 after a carry
-  const long long bits = (static_cast<long long>(k + 62 - lz) << 52) + static_cast<long long>(a);
-  return __longlong_as_double(bits | (r & (1ll << 63)));
+  constexpr long long M28 = (1ll << 28) - 1;
+  // the sum as hi 2^64 + lo in units of 2^-8, then its size
+  const long long mid = s.hl + (s.ll >> 28);
+  long long hi = s.hh + (mid >> 28);
+  unsigned long long lo = static_cast<unsigned long long>((mid & M28) << 28 | (s.ll & M28)) << 8;
+  const long long sign = hi & (1ll << 63);
+  if (hi < 0) {
+    lo = -lo;
+    hi = ~hi + (lo == 0);
+  }
+  if (hi == 0) {
+    if (lo == 0) return 0.0;
+    hi = lo >> 8;
+    lo = 0;
+    k -= 56;
+  }
+  const int lz = __clzll(hi);
+  const unsigned long long top = (static_cast<unsigned long long>(hi) << lz) | (lo >> 1 >> (63 - lz));
+  const unsigned long long m = (top >> 11) + ((top >> 10) & 1);  // 53 bits, or 2^53
+  const long long bits = (static_cast<long long>(k + 91 - lz) << 52) + static_cast<long long>(m);
+  return __longlong_as_double(bits | sign);
 }
 
 template <int N, int MODE, bool MEDIA>
@@ -154,20 +193,28 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
   // interior column of the own node, -1 at a vertex node
   const int ci = (i == 0 || i == N || i == Np - 1) ? -1 : i < N ? i - 1 : i - 2;
 
-  int2* tab = reinterpret_cast<int2*>(smem);  // Dr [NI][Np], Ds [NI][Np], LIFT [Nafp][Np]
-  unsigned char* stages = smem + 8 * L::TABLE;
+  // the table (f64_table_ints)
+  int4* tab4 = reinterpret_cast<int4*>(smem);
+  int2* tab2 = reinterpret_cast<int2*>(tab4 + NI * Np);
+  int2* tabl = tab2 + NI * Np;
+  int* tablz = reinterpret_cast<int*>(tabl + Nafp * Np);
+  unsigned char* stages = smem + 4 * L::TABLE;
   const int SB = L::stage_bytes(E);
-  int2* ops = reinterpret_cast<int2*>(stages + 2 * SB);  // per element: z, A, B [NI], f, g [Nafp]
-  double* dif = reinterpret_cast<double*>(ops + E * L::OPS);  // [E][3][2]
+  const bool two = !MEDIA && p.alpha != 1.0;  // a second flux scalar
+  const int NF = two ? 2 * Nafp : Nafp;
+  // per element and column {z x, y, A x, y}, {B x, y, z z, A z}; per face node {x, y, z}
+  int4* vol = reinterpret_cast<int4*>(stages + 2 * SB);
+  int4* flx = vol + 2 * NI * E;
+  double* dif = reinterpret_cast<double*>(flx + NF * E);      // [E][3][2]
   double* lin = dif + 6 * E;                                  // [3][E]
   int* mx = reinterpret_cast<int*>(lin + 3 * E);              // [2][E][4]
+  int* volb = mx + 8 * E;                                     // B z [E][NI]
 
   const int K = static_cast<int>(p.K);
   const int nblk = (K + E - 1) / E;
   const int G = gridDim.x, b0 = blockIdx.x;
   const int niter = b0 < nblk ? (nblk - 1 - b0) / G + 1 : 0;
   const int64_t fs = p.fstride;
-  const bool two = !MEDIA && p.alpha != 1.0;  // a second flux scalar
 
   auto stage = [&](int it) { return reinterpret_cast<double*>(stages + (it & 1) * SB); };
   auto codes = [&](int it) {
@@ -199,10 +246,10 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
   if (niter > 0) issue_geo(0);
   {
     const int4* src = static_cast<const int4*>(p.tc_op);
-    for (int c = t; c < L::TABLE / 2; c += NT) cp_async16(tab + 2 * c, src + c);
+    for (int c = t; c < L::TABLE / 4; c += NT) cp_async16(tab4 + c, src + c);
   }
   // powers of two of this node's rows of Dr and Ds, and of LIFT
-  const int2 scale = __ldg(static_cast<const int2*>(p.tc_op) + L::TABLE + i);
+  const int2 scale = __ldg(static_cast<const int2*>(p.tc_op) + L::TABLE / 2 + i);
   const double lam2 = __ldg(p.lam + i), lam3 = __ldg(p.lam + Np + i);
   for (int c = t; c < 8 * E; c += NT) mx[c] = 0;
 
@@ -328,23 +375,28 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
 
     // ---- 2: fixed-point operands
     auto slot = [&](double v, int size) {
-      if (size == 0) return make_int2(0, 0);
+      if (size == 0) return F64Limbs{0, 0, 0};
       return f64_fixed(size) ? f64_limbs(v, size >> 20)
-                             : make_int2(__double2hiint(v), __double2loint(v));
+                             : F64Limbs{__double2hiint(v), __double2loint(v), 0};
     };
     if (valid && ci >= 0) {
-      int2* o = ops + e * L::OPS + ci;
-      o[0] = slot(z, m[4 * e]);
-      o[NI] = slot(A, m[4 * e + 1]);
-      o[2 * NI] = slot(B, m[4 * e + 1]);
+      const F64Limbs lz = slot(z, m[4 * e]), la = slot(A, m[4 * e + 1]), lb = slot(B, m[4 * e + 1]);
+      int4* o = vol + 2 * (e * NI + ci);
+      o[0] = make_int4(lz.x, lz.y, la.x, la.y);
+      o[1] = make_int4(lb.x, lb.y, lz.z, la.z);
+      volb[e * NI + ci] = lb.z;
     }
 #pragma unroll
     for (int u = 0; u < TPT; ++u) {
       const int ee = task_e[u];
       if (ee < E && k0 + ee < K) {
-        int2* o = ops + ee * L::OPS + 3 * NI + task_j[u];
-        o[0] = slot(fv[u], m[4 * ee + 2]);
-        if (two) o[Nafp] = slot(gv[u], m[4 * ee + 3]);
+        int4* o = flx + ee * NF + task_j[u];
+        const F64Limbs lf = slot(fv[u], m[4 * ee + 2]);
+        o[0] = make_int4(lf.x, lf.y, lf.z, 0);
+        if (two) {
+          const F64Limbs lg = slot(gv[u], m[4 * ee + 3]);
+          o[Nafp] = make_int4(lg.x, lg.y, lg.z, 0);
+        }
       }
     }
     cp_async_wait<0>();
@@ -353,7 +405,17 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
 
     // ---- 3: products, chain rule, update
     if (valid) {
-      const int2* o = ops + e * L::OPS;
+      const int4* vo = vol + 2 * e * NI;
+      const int* vb = volb + e * NI;
+      const int4* fo = flx + e * NF;
+      auto lift = [&](int j) {
+        const int2 h = tabl[j * Np + i];
+        return F64Limbs{h.x, h.y, tablz[j * Np + i]};
+      };
+      auto flux = [&](int j) {
+        const int4 h = fo[j];
+        return F64Limbs{h.x, h.y, h.z};
+      };
       const int sz = m[4 * e], sab = m[4 * e + 1], sf = m[4 * e + 2], sgg = m[4 * e + 3];
       const bool fixed = f64_fixed(sz) && f64_fixed(sab) && f64_fixed(sf) && f64_fixed(sgg);
       double zr, zs, c, lf[3], lsum;  // lf: LIFT of the H rows' scalar per face
@@ -361,14 +423,15 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
         F64Sum szr, szs, sc;
 #pragma unroll UNROLL
         for (int k = 0; k < NI; ++k) {
-          const int2 dr = tab[k * Np + i], ds = tab[(NI + k) * Np + i];
-          const int2 vz = o[k];
+          const int4 d = tab4[k * Np + i], u = vo[2 * k], w = vo[2 * k + 1];
+          const int2 dz = tab2[k * Np + i];
+          const F64Limbs dr = {d.x, d.y, dz.x}, ds = {d.z, d.w, dz.y};
+          const F64Limbs vz = {u.x, u.y, w.z};
           szr.term(dr, vz);
           szs.term(ds, vz);
-          sc.term(dr, o[NI + k]);
-          sc.term(ds, o[2 * NI + k]);
+          sc.term(dr, F64Limbs{u.z, u.w, w.w});
+          sc.term(ds, F64Limbs{w.x, w.y, vb[k]});
         }
-        const int2* lt = tab + 2 * NI * Np + i;
         const int kz = (sz >> 20) + scale.x, kab = (sab >> 20) + scale.x;
         zr = f64_value(szr, kz);
         zs = f64_value(szs, kz);
@@ -381,7 +444,7 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
 #pragma unroll UNROLL
           for (int jj = 0; jj < Nfp; ++jj) {
             const int j = f * Nfp + jj;
-            face.term(lt[j * Np], o[3 * NI + j]);
+            face.term(lift(j), flux(j));
           }
           lf[f] = f64_value(face, kf);
           all.add(face);
@@ -395,27 +458,30 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
 #pragma unroll UNROLL
             for (int jj = 0; jj < Nfp; ++jj) {
               const int j = f * Nfp + jj;
-              face.term(lt[j * Np], o[3 * NI + Nafp + j]);
+              face.term(lift(j), flux(Nafp + j));
             }
             lf[f] = f64_value(face, kg);
           }
         }
       } else {
         // some operand has no fixed-point form: all of the element's in FP64
-        auto at = [&](int k, int size) {
-          if (!f64_fixed(size)) return __hiloint2double(o[k].x, o[k].y);
+        auto at = [](int x, int y, int lo, int size) {
+          if (!f64_fixed(size)) return __hiloint2double(x, y);
+          const double low = static_cast<double>(y) * 268435456.0 + lo;
           return size == 0 ? 0.0
-                           : scalbn(static_cast<double>(o[k].x) * 268435456.0 + o[k].y,
-                                    (size >> 20) - 1077);
+                           : scalbn(static_cast<double>(x) * 72057594037927936.0 + low,
+                                    (size >> 20) - 1106);
         };
         zr = zs = c = lsum = 0.0;
 #pragma unroll 1
         for (int k = 0; k < NI; ++k) {
           const int col = i * Np + (k < N - 1 ? k + 1 : k + 2);
           const double dr = __ldg(p.Dr + col), ds = __ldg(p.Ds + col);
-          zr += dr * at(k, sz);
-          zs += ds * at(k, sz);
-          c += dr * at(NI + k, sab) + ds * at(2 * NI + k, sab);
+          const int4 u = vo[2 * k], w = vo[2 * k + 1];
+          const double vz = at(u.x, u.y, w.z, sz);
+          zr += dr * vz;
+          zs += ds * vz;
+          c += dr * at(u.z, u.w, w.w, sab) + ds * at(w.x, w.y, vb[k], sab);
         }
 #pragma unroll
         for (int f = 0; f < 3; ++f) {
@@ -423,9 +489,11 @@ __global__ void __launch_bounds__(f64_max_elems(N) * Order<N>::Np, f64_ctas(N))
 #pragma unroll 1
           for (int jj = 0; jj < Nfp; ++jj) {
             const int j = f * Nfp + jj;
-            const double l = __ldg(p.LIFT + i * Nafp + j), v = at(3 * NI + j, sf);
+            const double l = __ldg(p.LIFT + i * Nafp + j);
+            const int4 a = fo[j], b = fo[two ? Nafp + j : j];
+            const double v = at(a.x, a.y, a.z, sf);
             lsum += l * v;
-            lf[f] += l * (two ? at(3 * NI + Nafp + j, sgg) : v);
+            lf[f] += l * (two ? at(b.x, b.y, b.z, sgg) : v);
           }
         }
       }
@@ -481,11 +549,11 @@ cudaError_t launch_f64_mode(const StageArgs<double>& args, int num_sms, cudaStre
   cudaError_t err = configure_once_per_device(configured, [] {
     cudaError_t e = cudaFuncSetAttribute(dg_stage_f64_kernel<N, MODE, MEDIA>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         L::smem_bytes(EMAX));
+                                         L::smem_bytes(EMAX, !MEDIA));
     int nb = 0;
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, dg_stage_f64_kernel<N, MODE, MEDIA>,
-                                                        EMAX * L::Np, L::smem_bytes(EMAX));
+                                                        EMAX * L::Np, L::smem_bytes(EMAX, false));
     if (e == cudaSuccess) blocks_per_sm.store(nb > 0 ? nb : 1);
     return e;
   });
@@ -495,7 +563,7 @@ cudaError_t launch_f64_mode(const StageArgs<double>& args, int num_sms, cudaStre
   int64_t grid = static_cast<int64_t>(blocks_per_sm.load()) * num_sms;
   if (grid > nblk || E < EMAX) grid = nblk;
   return launch_chained(dg_stage_f64_kernel<N, MODE, MEDIA>, static_cast<unsigned>(grid),
-                        E * L::Np, L::smem_bytes(E), stream, args, E);
+                        E * L::Np, L::smem_bytes(E, !MEDIA && args.alpha != 1.0), stream, args, E);
 }
 
 template <int N, bool MEDIA>

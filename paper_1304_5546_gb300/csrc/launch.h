@@ -77,12 +77,12 @@ constexpr int kSmallNone = 0, kSmallNodes = 1, kSmallElems = 2;
 // FP64 stage kernel (kernels_f64.cuh).  Most elements per block: threads E Np
 // just under a whole number of warps (a partial warp costs the FP64 pipe as
 // much as a full one).  GB300, us per LSRK step, products in FP64 (a thread
-// per node, the form before) / in fixed point: N = 1, K = 180,000 640 / 309;
-// 2, 80,000 631 / 329; 3, 45,000 678 / 308; 4, 45,000 1200 / 406; 5, 101,250
-// 4020 / 1290 (FP64 pipe 0.61 busy by the counter, 0.78 of what back-to-back
-// FMAs reach); 6, 20,000 1267 / 371; 7, 20,000 1965 / 541; with a
-// permittivity 1901 / 560.  Small: N = 4, K = 128 82 / 34; N = 7, K = 128 165
-// / 40.
+// per node, the form before) / in fixed point: N = 1, K = 180,000 640 / 320;
+// 2, 80,000 631 / 354; 3, 45,000 678 / 337; 4, 45,000 1200 / 439; 5, 101,250
+// 4020 / 1453; 6, 20,000 1267 / 472; 7, 20,000 1965 / 695.  Small: N = 4, K =
+// 128 82 / 37.  (Others at N = 5, 6 / 12 elements 1510 / 1590 beside 1509 for 9
+// with three columns a step; N = 6, 6 / 9 506 / 485 beside 484; N = 7, 4 / 6 / 8
+// 799 / 748 / 774 beside 729.)
 __host__ __device__ constexpr int f64_max_elems(int N) {
   return N == 1 ? 64 : N == 2 ? 16 : N == 3 ? 16 : N == 4 ? 17 : N == 5 ? 9 : N == 6 ? 8 : 7;
 }
@@ -258,12 +258,12 @@ cudaError_t launch_stage_tc(const StageArgs<float>& args, int mode, int num_sms,
                             cudaStream_t stream);
 
 // FP64 path (see kernels_f64.cuh).  tc_op of its StageArgs: Dr and Ds without
-// the vertex nodes' columns, and LIFT, in fixed point -- limb pairs
-// [column][node] of 8 bytes, then per node a pair with the powers of two of
-// its rows' scales (of Dr and Ds, of LIFT); built by f64_operator_table
-// (api.cu).
-__host__ __device__ constexpr int f64_table_pairs(int N) {  // rounded up to 16 bytes
-  return ((2 * (tc_np(N) - 3) + 3 * (N + 1)) * tc_np(N) + 1) / 2 * 2;
+// the vertex nodes' columns, and LIFT, in fixed point of three limbs x, y, z
+// (f64_operator_table, api.cu), all [column][node]: {Dr x, Dr y, Ds x, Ds y},
+// {Dr z, Ds z}, {LIFT x, LIFT y}, {LIFT z}; from the next 16 bytes on, per
+// node, the powers of two of its rows' scales (of Dr and Ds, of LIFT).
+__host__ __device__ constexpr int f64_table_ints(int N) {  // in whole 16 bytes
+  return (3 * (2 * (tc_np(N) - 3) + 3 * (N + 1)) * tc_np(N) + 3) / 4 * 4;
 }
 template <int N>
 cudaError_t launch_stage_f64(const StageArgs<double>& args, bool media, int mode, int num_sms,

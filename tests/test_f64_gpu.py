@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 import oracle as O
-from synth import jittered_delaunay_mesh, random_permittivity
+from synth import jittered_delaunay_mesh, random_permittivity, square_grid_mesh
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-12
@@ -97,3 +97,85 @@ def test_non_finite_values_stay_where_they_reach(P, N, bad):
     np.testing.assert_array_equal(got[:, rest], clean[:, rest])
     assert not np.isfinite(got[:2, k]).any()
     s.close()
+
+
+def _rhs_and_size(P, s, q, alpha, eps):
+    """The right-hand side from the operator's own tables and geometry in
+    extended precision, and the sum of the absolute values of its terms."""
+    LD = np.longdouble
+    R, G = P.dg_get_reference(s.op), P.dg_get_geometry(s.op)
+    vM, vP = P.dg_get_maps(s.op)
+    wall = vM == vP
+    N, Nfp = s.N, R["Fmask"].shape[1]
+    q = q.astype(LD)
+    out = []
+    for absolute in (False, True):
+        sg = (lambda v: np.abs(v)) if absolute else (lambda v: v)
+        minus = LD(1 if absolute else -1)  # the sign of a subtracted term
+        Dr, Ds, L = (sg(R[k].astype(LD)) for k in ("Dr", "Ds", "LIFT"))
+        rx, ry, sx, sy = (sg(G[k].astype(LD))[:, None] for k in ("rx", "ry", "sx", "sy"))
+        nx, ny, F = (sg(np.repeat(G[k].astype(LD), Nfp, axis=1)) for k in ("nx", "ny", "Fscale"))
+        u = [sg(c) for c in q]
+        # a field is its linear interpolant (derivatives half the vertex
+        # differences) and the rest
+        lam2, lam3 = ((1 + R[k].astype(LD)) / 2 for k in ("r", "s"))
+        rest, gr, gs = [], [], []
+        for c in u:
+            v1, d2, d3 = c[:, :1], c[:, N:N + 1] + minus * c[:, :1], c[:, -1:] + minus * c[:, :1]
+            rest.append(c + minus * v1 + minus * (d2 * lam2 + d3 * lam3))
+            gr.append(d2 / 2)
+            gs.append(d3 / 2)
+        dx, dy, dz = (c.ravel()[vM] + minus * c.ravel()[vP] for c in u)
+        dx, dy = (np.where(wall, LD(0), d) for d in (dx, dy))
+        dz = np.where(wall, 2 * u[2].ravel()[vM], dz)
+        Ht = ny * dx + minus * nx * dy
+        if eps is None:
+            fh, fz = F / 2 * (LD(alpha) * Ht + minus * dz), F / 2 * (Ht + minus * LD(alpha) * dz)
+            zm = sH = sE = LD(1)
+        else:
+            Z = 1 / np.sqrt(eps.astype(LD))
+            zM, zP = np.repeat(Z[:, None], 3 * Nfp, axis=1), Z[vP // s.Np]
+            fh = fz = F / (zM + zP) * (zP * Ht + minus * dz)
+            zm, sH, sE = zM, LD(1), 1 / eps.astype(LD)[:, None]
+        hx, hy, ez = rest
+        zr, zs = ez @ Dr.T + gr[2], ez @ Ds.T + gs[2]
+        A, B = rx * hy + minus * ry * hx, sx * hy + minus * sy * hx
+        lin = rx * gr[1] + minus * ry * gr[0] + sx * gs[1] + minus * sy * gs[0]
+        out.append(np.stack([
+            sH * (minus * (ry * zr + sy * zs) + minus * (zm * ny * fh) @ L.T),
+            sH * (rx * zr + sx * zs + (zm * nx * fh) @ L.T),
+            sE * (A @ Dr.T + B @ Ds.T + lin + fz @ L.T)]))
+    return out
+
+
+# Every component to within 32 roundings (2^-53) of the sum of its own terms'
+# sizes: a term meets at most 16 on its way (operands 5, coefficients 4,
+# product 1, chain rule, update of the sum and row scale 6).  Bubbles with
+# entries over nine decades on zero vertices, which deflation leaves as they
+# are; and one element far above its neighbours, on axis-aligned faces: where
+# a normal's component is zero, a large flux has no part in that row.
+@pytest.mark.parametrize("form", ["upwind", "alpha", "media"])
+@pytest.mark.parametrize("N", range(1, 8))
+@pytest.mark.parametrize("kind", ["bubbles", "one large"])
+def test_small_components_keep_their_precision(P, kind, N, form):
+    mesh = jittered_delaunay_mesh(6, seed=4) if kind == "bubbles" else square_grid_mesh(5, 5)
+    s = P.Solver(*mesh, N=N, precision="fp64",
+                 eps=random_permittivity(mesh[2].shape[0], seed=2) if form == "media" else None)
+    alpha = 0.25 if form == "alpha" else 1.0
+    if form == "alpha":
+        P.dg_operator_set_alpha(s.op, alpha)
+    rng = np.random.default_rng(N)
+    shape = (3, s.K, s.Np)
+    q = rng.uniform(0.5, 1, shape) * rng.choice([-1.0, 1.0], shape)
+    if kind == "bubbles":
+        q *= 10.0 ** rng.uniform(-9, 0, shape)
+        q[:, :, [0, N, s.Np - 1]] = 0.0
+    else:
+        q *= 1e-8
+        q[:, 22] *= 1e8
+    eps = random_permittivity(s.K, seed=2) if form == "media" else None
+    want, size = _rhs_and_size(P, s, q, alpha, eps)
+    got = _rhs(P, s, q)
+    s.close()
+    assert (np.abs(got - want) <= 32 * 2.0 ** -53 * size).all(), \
+        float((np.abs(got - want)[size > 0] / size[size > 0]).max() * 2 ** 53)
