@@ -306,10 +306,12 @@ dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, double* ms_tc,
  * dg_operator_tune).  On a large mesh at N = 3..5 the default is a kernel
  * with one GEMM row per element and blocks of 128; the sizes of the other
  * tensor-core kernel (80 and 40, 40 and 80, 40) select that one; on a small
- * mesh, where the default is a CUDA-core kernel, they do so too (at N <= 2, 32
- * selects the element-thread kernel).  The blocks are a kernel's unit of work:
- * each CTA of the persistent launch walks blocks of this many consecutive
- * elements.
+ * mesh, where the default is a CUDA-core kernel, they do so too, and the size
+ * that dg_operator_kernel reports there selects that kernel again.  At N = 1
+ * and 2, 32 always selects the element-thread kernel: at N = 2 the node-thread
+ * kernel of small meshes has blocks of 32 as well, and 0 selects it.  The
+ * blocks are a kernel's unit of work: each CTA of the persistent launch walks
+ * blocks of this many consecutive elements.
  * Results do not depend on the size beyond rounding.  With face pairs on,
  * the default size is used.
  * Errors: DG_ERR_ARG (NULL, a size the operator's kernel does not have). */

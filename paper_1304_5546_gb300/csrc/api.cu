@@ -535,11 +535,15 @@ int kernel_block_elems(const dg_op* op, int alt) {
   return dgw::simt_block_elems(op->N);
 }
 
+// Elements per block of the kernel of small meshes that the set-up chose.
+int small_block_elems(const dg_op* op) {
+  return op->small == dgw::kSmallElems ? 32 : dgw::simt_block_elems(op->N);
+}
+
 // The same with the kernels of large and of small meshes where the operator
 // runs them.
 int block_elems(const dg_op* op, int alt) {
-  if (op->precision == DG_FP32 && runs_small(op))
-    return op->small == dgw::kSmallElems ? 32 : dgw::simt_block_elems(op->N);
+  if (op->precision == DG_FP32 && runs_small(op)) return small_block_elems(op);
   return op->precision == DG_FP32 && runs_er(op) ? dgw::kErElems : kernel_block_elems(op, alt);
 }
 
@@ -1062,7 +1066,9 @@ extern "C" dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems) {
   const bool alt_ok = op->precision == DG_FP32 && op->use_tc && !op->use_ept &&
                       op->tc_prec == dgw::kTcTf32x3 && tc_has_alt_n(op->N);
   const int def = kernel_block_elems(op, 0), alt = alt_ok ? kernel_block_elems(op, 1) : def;
-  if (elems == 0 || (op->use_er && elems == dgw::kErElems)) {
+  const bool er_ok = op->use_er && op->use_tc && !op->use_ept;
+  const int small = op->small == dgw::kSmallNone ? def : small_block_elems(op);
+  if (elems == 0 || (er_ok && elems == dgw::kErElems)) {
     op->tc_alt = 0;
     op->er_off = op->small_off = false;
   } else if (elems == def) {
@@ -1071,10 +1077,16 @@ extern "C" dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems) {
   } else if (alt_ok && elems == alt) {
     op->tc_alt = 1;
     op->small_off = true;
+  } else if (elems == small) {
+    op->tc_alt = 0;
+    op->small_off = false;
   } else {
+    std::string sizes = std::to_string(def);
+    if (alt_ok) sizes += " or " + std::to_string(alt);
+    if (er_ok) sizes += " or " + std::to_string(dgw::kErElems);
+    if (small != def) sizes += " or " + std::to_string(small);
     return fail(DG_ERR_ARG, "%s: %d elements per block is not a size of this operator's kernel "
-                "(%d%s%s)", where, elems, def, alt_ok ? " or " : "",
-                alt_ok ? std::to_string(alt).c_str() : "");
+                "(%s)", where, elems, sizes.c_str());
   }
   return DG_OK;
 }

@@ -50,3 +50,25 @@ def test_partition_runs_the_kernel_that_was_set(P, N, elems, media):
     P.dg_sync_check(s.op)
     assert torch.equal(s.view(got), s.view(want))
     s.close()
+
+
+# the reported size keeps the kernel, on either side of every line of the
+# dispatch; N = 2's node threads and element threads both have blocks of 32
+@pytest.mark.parametrize("K", [100, 9000, 25000, 40000])
+@pytest.mark.parametrize("N", range(1, 8))
+def test_reported_block_size_is_accepted(P, N, K):
+    s = P.Solver(*_mesh(K), N=N)
+    first = s.kernel()
+    P.dg_operator_set_block_elems(s.op, first[1])
+    assert s.kernel() == (("element threads", 32) if N == 2 else first)
+    other = {1: 32, 2: 32, 3: 40, 4: 80, 5: 40, 6: 40, 7: 40}[N]
+    for size in (other, first[1]):  # away and back
+        P.dg_operator_set_block_elems(s.op, size)
+        assert s.kernel()[1] == size
+    assert s.kernel() == (("element threads", 32) if N == 2 else first)
+    P.dg_operator_set_block_elems(s.op, 0)
+    assert s.kernel() == first
+    with pytest.raises(P.DGError) as ex:
+        P.dg_operator_set_block_elems(s.op, 20)
+    assert ex.value.status == P._lib.DG_ERR_ARG
+    s.close()
