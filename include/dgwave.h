@@ -286,24 +286,27 @@ dg_status dg_get_maps(const dg_op* op, int64_t* vmapM, int64_t* vmapP);
  *   - the tensor-core kernel (3xTF32) in its default element-block size;
  *   - the same in its alternative size where there is one (40 elements at
  *     N = 1..3, where the default is 80; 80 at N = 4, where it is 40);
+ *   - the kernel of large meshes at N = 3..5 with blocks of 128, where the
+ *     set-up chose it (without face pairs; alpha = 1 or a permittivity);
  *   - unless DG_SETUP_TC, the CUDA cores: the node-thread kernel, and the
  *     element-thread kernel at N <= 5.
  * Writes the milliseconds per launch of the fastest tensor-core candidate
  * and of the fastest CUDA-core candidate (NULL outputs skipped; -1 where not
  * timed).  Operators whose set-up fixed the kernel and products (FP64,
  * DG_SETUP_SIMT, DG_SETUP_ELEMENT_THREADS, DG_SETUP_TC_*) are left as they
- * are.  dg_operator_kernel
- * reports the choice.  Call it before stepping, not while calls on the
- * operator are in flight.
+ * are.  dg_operator_kernel reports the choice, and
+ * dg_operator_set_block_elems(op, 0) takes it back.  Call it before stepping,
+ * not while calls on the operator are in flight.
  * Errors: DG_ERR_ARG (NULL, reps < 1), DG_ERR_NO_DEVICE, DG_ERR_OOM,
  * DG_ERR_CUDA.                                                             */
 dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, double* ms_tc,
                            double* ms_cuda_cores);
 
 /* dg_operator_set_block_elems: the element-block size of the operator's
- * kernel for later calls: 0 or the default size, or the tensor-core
+ * kernel for later calls: the default size, or the tensor-core
  * kernel's alternative size where it has one (3xTF32 products; see
- * dg_operator_tune).  On a large mesh at N = 3..5 the default is a kernel
+ * dg_operator_tune), or 0: the kernel and size that the set-up chose, whatever
+ * was set or tuned since.  On a large mesh at N = 3..5 the default is a kernel
  * with one GEMM row per element and blocks of 128; the sizes of the other
  * tensor-core kernel (80 and 40, 40 and 80, 40) select that one; on a small
  * mesh, where the default is a CUDA-core kernel, they do so too, and the size

@@ -433,12 +433,13 @@ cudaError_t launch_order_ept(const dg_op* op, const dgw::StageArgs<float>& a, in
   }
 }
 
-// The operator's hot-path calls run the element-row kernel (of an operator
-// on the tensor cores; without face pairs, and with alpha = 1 in a uniform
-// medium).
+// The operator has the element-row kernel and its settings allow it (no face
+// pairs, and alpha = 1 in a uniform medium); its hot-path calls run it.
+bool can_er(const dg_op* op) {
+  return op->use_er && !op->face_pairs && (op->media() || op->alpha == 1.0);
+}
 bool runs_er(const dg_op* op) {
-  return op->use_er && !op->er_off && op->use_tc && !op->use_ept && !op->tc_alt &&
-         !op->face_pairs && (op->media() || op->alpha == 1.0);
+  return can_er(op) && !op->er_off && op->use_tc && !op->use_ept && !op->tc_alt;
 }
 
 // They run the CUDA-core kernel of small meshes (small_kernel below).
@@ -728,6 +729,8 @@ dg_status operator_setup(const dg_mesh* mesh, int32_t N, const double* eps, int3
                  (N >= 2 || variants != 0 || (flags & DG_SETUP_TC));
     op->use_ept = (flags & DG_SETUP_ELEMENT_THREADS) ||
                   (precision == DG_FP32 && !(flags & chosen_kernels) && N <= 2);
+    op->setup_tc = op->use_tc;
+    op->setup_ept = op->use_ept;
     op->tc_prec = (flags & DG_SETUP_TC_TF32)    ? dgw::kTcTf32
                   : (flags & DG_SETUP_TC_BF16)  ? dgw::kTcBf16
                   : (flags & DG_SETUP_TC_BF16X3) ? dgw::kTcBf16x3
@@ -971,21 +974,24 @@ extern "C" dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, dou
                         DG_SETUP_ELEMENT_THREADS;
   if (op->precision != DG_FP32 || (op->flags & fixed)) return DG_OK;  // nothing to choose
   // candidates: tensor cores (3xTF32) in the default and, where there is one,
-  // the alternative element-block size; unless DG_SETUP_TC, the CUDA cores:
-  // the node-per-thread kernel, and the element-thread kernel where the
-  // operator has its tables (N <= kEptMaxN)
+  // the alternative element-block size, and the element-row kernel where the
+  // operator can run it; unless DG_SETUP_TC, the CUDA cores: the
+  // node-per-thread kernel, and the element-thread kernel where the operator
+  // has its tables (N <= kEptMaxN).  A small mesh's kernel is one of these two.
   struct Cand {
     bool tc;
     int alt;
-    bool ept;
-  } cand[4];
+    bool ept, er_off;
+  } cand[5];
   int nc = 0;
-  cand[nc++] = {true, 0, false};
-  if (tc_has_alt_n(op->N)) cand[nc++] = {true, 1, false};
+  const bool off = can_er(op) || op->er_off;  // of the candidates beside the element-row kernel
+  cand[nc++] = {true, 0, false, off};
+  if (tc_has_alt_n(op->N)) cand[nc++] = {true, 1, false, off};
+  if (can_er(op)) cand[nc++] = {true, 0, false, false};
   if (!(op->flags & DG_SETUP_TC)) {
-    cand[nc++] = {false, 0, false};
+    cand[nc++] = {false, 0, false, off};
     if (op->ept_ops.size() == static_cast<size_t>(dgw::ept_ops_floats(op->N)))
-      cand[nc++] = {false, 0, true};
+      cand[nc++] = {false, 0, true, off};
   }
   if (nc < 2) return DG_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -1009,14 +1015,18 @@ extern "C" dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, dou
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  const bool was_tc = op->use_tc, was_ept = op->use_ept;
-  const int was_alt = op->tc_alt, was_small = op->small;
-  op->small = dgw::kSmallNone;  // its kernels are among the candidates
-  float ms[4] = {0.f, 0.f, 0.f, 0.f};
+  const Cand was = {op->use_tc, op->tc_alt, op->use_ept, op->er_off};
+  const bool was_small_off = op->small_off;
+  op->small_off = true;
+  auto take = [&](const Cand& c) {
+    op->use_tc = c.tc;
+    op->tc_alt = c.alt;
+    op->use_ept = c.ept;
+    op->er_off = c.er_off;
+  };
+  float ms[5] = {};
   for (int v = 0; v < nc && err == cudaSuccess; ++v) {
-    op->use_tc = cand[v].tc;
-    op->tc_alt = cand[v].alt;
-    op->use_ept = cand[v].ept;
+    take(cand[v]);
     dgw::StageArgs<float> a = base_args<float>(op);
     a.qin = buf;
     a.qout = buf + 3 * op->fstride;
@@ -1037,18 +1047,14 @@ extern "C" dg_status dg_operator_tune(dg_op* op, int32_t reps, void* stream, dou
   cudaFree(buf);
   op->launches.fetch_add(nc * (reps + 1), std::memory_order_relaxed);
   if (err != cudaSuccess) {
-    op->use_tc = was_tc;
-    op->tc_alt = was_alt;
-    op->use_ept = was_ept;
-    op->small = was_small;
+    take(was);
+    op->small_off = was_small_off;
     return cuda_fail(err, "dg_operator_tune");
   }
   int best = 0;
   for (int v = 1; v < nc; ++v)
     if (ms[v] < ms[best]) best = v;
-  op->use_tc = cand[best].tc;
-  op->tc_alt = cand[best].alt;
-  op->use_ept = cand[best].ept;
+  take(cand[best]);
   double best_tc = -1.0, best_cc = -1.0;
   for (int v = 0; v < nc; ++v) {
     double& b = cand[v].tc ? best_tc : best_cc;
@@ -1068,7 +1074,12 @@ extern "C" dg_status dg_operator_set_block_elems(dg_op* op, int32_t elems) {
   const int def = kernel_block_elems(op, 0), alt = alt_ok ? kernel_block_elems(op, 1) : def;
   const bool er_ok = op->use_er && op->use_tc && !op->use_ept;
   const int small = op->small == dgw::kSmallNone ? def : small_block_elems(op);
-  if (elems == 0 || (er_ok && elems == dgw::kErElems)) {
+  if (elems == 0) {  // what the setup chose
+    op->use_tc = op->setup_tc;
+    op->use_ept = op->setup_ept;
+    op->tc_alt = 0;
+    op->er_off = op->small_off = false;
+  } else if (er_ok && elems == dgw::kErElems) {
     op->tc_alt = 0;
     op->er_off = op->small_off = false;
   } else if (elems == def) {

@@ -130,17 +130,20 @@ struct dg_op {
   int* d_status = nullptr; // kernel status word (bounded-wait expiry)
   void* d_tcop = nullptr;  // tensor-core operator tiles for FP32 (see tc_operator_tiles)
   // FP32 on the element-row kernel: what its setup chose (use_er), unless a
-  // block size of the other tensor-core kernel was asked for (er_off); its
-  // operator tiles and vertex-interpolant weights
+  // block size of the other tensor-core kernel was asked for, or
+  // dg_operator_tune chose that (er_off); its operator tiles and
+  // vertex-interpolant weights
   bool use_er = false, er_off = false;
   // FP32 on a small mesh: the kernel its setup chose instead (kSmall...),
-  // unless a block size of the kernel below was asked for (small_off)
+  // unless a block size of the kernel below was asked for, or dg_operator_tune
+  // chose (small_off)
   int small = 0;
   bool small_off = false;
   void* d_erop = nullptr;
   std::vector<float> er_weights;
   bool use_tc = false;     // FP32 products on the tensor cores
   bool use_ept = false;    // FP32: the element-thread kernel (takes precedence over use_tc)
+  bool setup_tc = false, setup_ept = false;  // both as the setup chose them (dg_operator_tune changes them)
   // FP32 operators of order <= kEptMaxN: the element-thread kernel's
   // reference tables (launch.h, ept_ops_floats)
   std::vector<float> ept_ops;

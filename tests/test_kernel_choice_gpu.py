@@ -72,3 +72,26 @@ def test_reported_block_size_is_accepted(P, N, K):
         P.dg_operator_set_block_elems(s.op, 20)
     assert ex.value.status == P._lib.DG_ERR_ARG
     s.close()
+
+
+# every kernel of the operator is a candidate, and 0 brings the set-up's back
+@pytest.mark.parametrize("N,K,cands", [(1, 300, 4), (2, 300, 4), (3, 300, 4), (3, 12000, 4),
+                                       (4, 300, 4), (5, 300, 3), (7, 300, 2), (3, 40000, 5),
+                                       (4, 40000, 5), (5, 40000, 4)])
+def test_tune_times_every_kernel_and_can_be_undone(P, N, K, cands):
+    s = P.Solver(*_mesh(K), N=N)
+    first = s.kernel()
+    assert (first[1] == 128) == (K == 40000)
+    n0 = P.dg_launch_count(s.op)
+    ms_tc, ms_cc = s.tune(reps=2)
+    assert ms_tc > 0 and ms_cc > 0
+    assert P.dg_launch_count(s.op) - n0 == 3 * cands
+    kernel, elems = s.kernel()
+    P.dg_operator_set_block_elems(s.op, elems)  # the choice can be set again
+    assert s.kernel() == (kernel, elems)
+    if kernel != "tensor cores" and elems != 128:
+        with pytest.raises(P.DGError):  # blocks of a kernel that does not run
+            P.dg_operator_set_block_elems(s.op, 128)
+    P.dg_operator_set_block_elems(s.op, 0)
+    assert s.kernel() == first
+    s.close()
