@@ -623,7 +623,8 @@ typedef struct dg_server dg_server;
 typedef struct dg_request_info {
   int32_t state;    /* DG_REQUEST_*                                        */
   int32_t status;   /* why a failed request failed (DG_ERR_OOM: it does not
-                       fit the pool of its order even when empty)          */
+                       fit the pool of its order even when empty;
+                       DG_ERR_CUDA: an error on the device)                */
   int32_t N;
   int64_t K;
   int64_t nsteps;   /* LSRK steps to the final time                        */
@@ -809,6 +810,12 @@ dg_status dg_sync_check(const dg_op* op, void* stream);
  * tests only.  Errors: DG_ERR_ARG (n < 0).                                 */
 dg_status dg_test_fail_alloc(int32_t n);
 int32_t dg_test_fail_alloc_pending(void);
+
+/* dg_test_result_state: the DG_REQUEST_* state a server gives a request whose
+ * result's event answers a query with this CUDA error code: done for 0,
+ * running while it is not ready, failed (DG_ERR_CUDA) for any other, so that
+ * nobody waits for a result that cannot come.  For tests only.             */
+int32_t dg_test_result_state(int32_t cuda_error);
 
 /* dg_test_wait_timeout: the timeout path, exercised without any fault.
  * Launches one right-hand-side pass of a tensor-core operator whose memory

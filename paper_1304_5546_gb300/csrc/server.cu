@@ -130,24 +130,34 @@ void finish(dg_server* s, Request* r, int32_t state, dg_status status) {
   s->cv_done.notify_all();
 }
 
-// requests whose results reached host memory
+// State of a request whose result's event was queried: still on its way, out,
+// or lost to an error on the device, which no later query would clear.
+int32_t result_state(cudaError_t query) {
+  return query == cudaSuccess         ? DG_REQUEST_DONE
+         : query == cudaErrorNotReady ? DG_REQUEST_RUNNING
+                                      : DG_REQUEST_FAILED;
+}
+
+// requests whose results reached host memory, or cannot any more
 void poll_finishing(dg_server* s) {
   for (size_t i = 0; i < s->finishing.size();) {
     Request* r = s->finishing[i];
-    if (cudaEventQuery(r->out_ev) != cudaSuccess) {
+    const int32_t state = result_state(cudaEventQuery(r->out_ev));
+    if (state == DG_REQUEST_RUNNING) {
       ++i;
       continue;
     }
     if (r->staged) {
       const int Np = r->op->Np;
-      std::memcpy(r->out, s->out_staging.ptr(r->staging_idx),
-                  3 * static_cast<size_t>(r->op->K) * Np * sizeof(float));
+      if (state == DG_REQUEST_DONE)
+        std::memcpy(r->out, s->out_staging.ptr(r->staging_idx),
+                    3 * static_cast<size_t>(r->op->K) * Np * sizeof(float));
       s->out_staging.unhold(r->staging_idx);
       r->staged = false;
     }
     s->spare_events.push_back(r->out_ev);
     r->out_ev = nullptr;
-    finish(s, r, DG_REQUEST_DONE, DG_OK);
+    finish(s, r, state, state == DG_REQUEST_DONE ? DG_OK : DG_ERR_CUDA);
     s->finishing[i] = s->finishing.back();
     s->finishing.pop_back();
   }
@@ -355,6 +365,10 @@ void worker_loop(dg_server* s) {
 
 // ============================================================ C ABI
 extern "C" double dg_server_clock(void) { return now_s(); }
+
+extern "C" int32_t dg_test_result_state(int32_t cuda_error) {
+  return result_state(static_cast<cudaError_t>(cuda_error));
+}
 
 extern "C" dg_status dg_server_create(const int64_t* capacity, int32_t flags, dg_server** out) {
   dgw::clear_error();
