@@ -662,8 +662,11 @@ dg_status dg_server_set_work_limit(dg_server* server, int64_t max_nodes);
  * from the host fields q0 (3 * K * Np floats in the layout of
  * dg_batch_set_fields with stride K * Np; NULL: zero fields; read at
  * admission, so it must stay valid until then) and writing the fields at T
- * to `out` (same layout; NULL: discard), host memory that must stay valid
- * until the request is done.  Returns at once with the request id.
+ * to `out` (same layout; NULL: discard), host memory that must stay mapped and
+ * writable until the request is done: where the device uses the host's page
+ * tables a kernel writes the fields there, elsewhere (and at an address that
+ * is not a multiple of 4) the host copies them from pinned memory.  Returns at
+ * once with the request id.
  * Errors: DG_ERR_ARG (NULL, not DG_FP32, T not positive, step count out
  * of range, server stopping), DG_ERR_OOM.                                  */
 dg_status dg_server_submit(dg_server* server, const dg_op* op, double T,
@@ -810,6 +813,13 @@ dg_status dg_sync_check(const dg_op* op, void* stream);
  * tests only.  Errors: DG_ERR_ARG (n < 0).                                 */
 dg_status dg_test_fail_alloc(int32_t n);
 int32_t dg_test_fail_alloc_pending(void);
+
+/* dg_test_host_touch: what a server does to the pages of a result before a
+ * kernel writes them: one byte of each page of [p, p + bytes) is read and
+ * written back.  The contents stay, nothing beside the range is accessed, and
+ * a page that the host may not write faults on the host.  For tests only.
+ * Errors: DG_ERR_ARG (NULL, bytes < 0).                                    */
+dg_status dg_test_host_touch(void* p, int64_t bytes);
 
 /* dg_test_result_state: the DG_REQUEST_* state a server gives a request whose
  * result's event answers a query with this CUDA error code: done for 0,

@@ -106,6 +106,7 @@ SIGNATURES = [
     ("dg_launch_count", c_i64, [c_void_p]),
     ("dg_test_wait_timeout", c_i32, [c_void_p, c_void_p]),
     ("dg_test_result_state", c_i32, [c_i32]),
+    ("dg_test_host_touch", c_i32, [c_void_p, c_i64]),
     ("dg_test_fail_alloc", c_i32, [c_i32]),
     ("dg_test_fail_alloc_pending", c_i32, []),
     ("dg_checkpoint_save", c_i32, [c_void_p, c_void_p, c_i64, c_i32, c_dbl, c_i64, ctypes.c_char_p]),

@@ -24,6 +24,7 @@
 // request only when none is running: plain one-at-a-time solves through the
 // same code, the baseline continuous batching is measured against.
 #include <cuda_runtime.h>
+#include <unistd.h>
 
 #include <atomic>
 #include <chrono>
@@ -78,7 +79,8 @@ struct dg_server {
   dg_batch* batch = nullptr;
   cudaStream_t stream = nullptr;
   // The device reads and writes pageable host memory through the host's page
-  // tables: a kernel writes the results where the caller wants them.
+  // tables: a kernel writes the results where the caller wants them, once the
+  // worker has touched their pages (host_touch).
   // Otherwise (and where `out` is not aligned to a float) they go through
   // pinned memory, from which the worker copies them at 14 GB/s, beside 170
   // over the link.  GB300, pinned / direct: 20 requests with 22 MB of results
@@ -250,6 +252,18 @@ void drop_cancelled(dg_server* s) {
   }
 }
 
+// One byte of every page of [p, p + bytes) read and written back by the host,
+// before a kernel stores there.  A page that the process may not write faults
+// here, in the worker, as a copy by the host does, and not on the device; and
+// pages that nobody has written yet come from the host's memory, as they do for
+// such a copy.
+void host_touch(void* p, size_t bytes) {
+  const size_t page = static_cast<size_t>(sysconf(_SC_PAGESIZE));
+  volatile unsigned char* b = static_cast<unsigned char*>(p);
+  for (size_t at = 0; at < bytes; at += page - (reinterpret_cast<uintptr_t>(p) + at) % page)
+    b[at] = b[at];
+}
+
 // requests at their final time: results out, range freed
 dg_status retire(dg_server* s) {
   for (size_t i = 0; i < s->running.size();) {
@@ -259,7 +273,10 @@ dg_status retire(dg_server* s) {
       continue;
     }
     dg_status st = DG_OK;
-    if (r->out && s->direct_out && reinterpret_cast<uintptr_t>(r->out) % sizeof(float) == 0) {
+    const bool direct =
+        r->out && s->direct_out && reinterpret_cast<uintptr_t>(r->out) % sizeof(float) == 0;
+    if (direct) {
+      host_touch(r->out, 3 * static_cast<size_t>(r->op->K) * r->op->Np * sizeof(float));
       st = dgw::batch_fields_to_host(s->batch, r->slot, static_cast<float*>(r->out), s->stream);
     } else if (r->out) {
       const int64_t n = r->op->K * r->op->Np;
@@ -286,6 +303,7 @@ dg_status retire(dg_server* s) {
     if (st != DG_OK) {
       if (r->staged) s->out_staging.unhold(r->staging_idx);
       r->staged = false;
+      if (direct) cudaStreamSynchronize(s->stream);  // nothing writes to `out` any more
       s->spare_events.push_back(r->out_ev);
       r->out_ev = nullptr;
       finish(s, r, DG_REQUEST_FAILED, st);
@@ -365,6 +383,13 @@ void worker_loop(dg_server* s) {
 
 // ============================================================ C ABI
 extern "C" double dg_server_clock(void) { return now_s(); }
+
+extern "C" dg_status dg_test_host_touch(void* p, int64_t bytes) {
+  dgw::clear_error();
+  if (!p || bytes < 0) return fail(DG_ERR_ARG, "dg_test_host_touch: NULL or bytes < 0");
+  host_touch(p, static_cast<size_t>(bytes));
+  return DG_OK;
+}
 
 extern "C" int32_t dg_test_result_state(int32_t cuda_error) {
   return result_state(static_cast<cudaError_t>(cuda_error));
