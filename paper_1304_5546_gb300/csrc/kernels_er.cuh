@@ -121,6 +121,9 @@ struct ErLayout {
   static constexpr int SMEM_BYTES = bytes(QS, RS, FBUF);
   static_assert(SMEM_BYTES <= SMAX && SMEM_BYTES > 118784, "one CTA per SM, which owns the TMEM");
   static_assert(AB * ACC + XB * 2 * XC <= 512, "tensor memory");
+  // an element group waits on mma_done of its own blocks and of the blocks XB
+  // before them: with one accumulator it sees every phase only if XB is odd
+  static_assert(AB == 2 || XB == 1, "every phase of mma_done seen by both element groups");
   static_assert(Np <= 32 && E == 128, "5-bit node table; element warps");
   static_assert(NZ % 16 == 0 && NF % 16 == 0 && NL % 16 == 0 && NZ <= 256 && Nfp <= KF, "UMMA shape");
   static_assert(QB % 128 == 0 && GB % 16 == 0 && OB % 128 == 0, "TMA chunks");
