@@ -451,8 +451,7 @@ cudaError_t launch_concurrent(dg_batch* b, int src, int stage, int reps, bool wh
 }
 
 // `count` launches of stage `stage` (reading buffer src) of order g on s, a
-// chain: each launch has a block for every CTA, so that each waits for the
-// launch before it.
+// chain: every CTA waits for the launch before it, with blocks or without.
 cudaError_t launch_chain(dg_batch* b, int g, int src, int stage, int count, cudaStream_t s) {
   cudaError_t err = cudaSuccess;
   for (int r = 0; r < count && err == cudaSuccess; ++r)

@@ -1503,12 +1503,17 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // SM striding over the order's block table; the orders' kernels run side by
 // side and the hardware gives SMs to whichever has CTAs waiting.  CTAs past
 // the order's block count (read from device memory, so that a captured
-// graph replays unchanged when problems join or leave) return at once.
+// graph replays unchanged when problems join or leave) return at once; in a
+// chain they too end only after the launch before, or a launch without blocks
+// would let the next one run beside that.
 template <int N, int MODE, bool ALT>
 __global__ void __launch_bounds__(kTcThreads, 1)
     dg_batch_order_kernel(const __grid_constant__ StageArgs<float> g) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  if (static_cast<int>(blockIdx.x) >= __ldg(g.nblocks)) return;
+  if (static_cast<int>(blockIdx.x) >= __ldg(g.nblocks)) {
+    chain_wait();
+    return;
+  }
   static_assert(TcLayout<N, kTcTf32x3, true, ALT>::THREADS == kTcThreads, "block size");
   tc_stage_body<N, MODE, kTcTf32x3, true, true, false, ALT, true>(g, blockIdx.x, gridDim.x, smem);
 }
