@@ -111,3 +111,32 @@ def test_partition_and_capture_are_bit_equal(P, N, media):
         torch.cuda.synchronize()
         assert torch.equal(s.view(q), s.view(want))
     P.dg_sync_check(s.op)
+
+
+# LIFT is one block-diagonal tile, whose zeros meet what a face's flux holds:
+# a value that is not finite must reach the elements that it reaches in the
+# other tensor-core kernel, whole, and no other element
+@pytest.mark.parametrize("media", [False, True])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("N", [3, 4, 5])
+def test_non_finite_values_stay_where_they_reach(P, N, bad, media):
+    mesh = _mesh(158, 83)
+    K = mesh[2].shape[0]
+    s = P.Solver(*mesh, N=N, eps=random_permittivity(K, seed=3) if media else None)
+    assert s.kernel() == ("tensor cores", 128)
+    q = np.random.default_rng(N).uniform(-1, 1, (3, K, s.Np))
+    run = lambda: s.to_numpy(s.rhs(s.from_numpy(q)))
+    clean = run()
+    ks = [0, 127, 128, 20000, K - 1]  # first and last of a block, and of the ragged one
+    for k, field in zip(ks, (2, 0, 1, 2, 2)):
+        q[field, k, 0] = bad
+    got = run()
+    P.dg_operator_set_block_elems(s.op, 80 if N == 3 else 40)
+    other = run()
+    hit = np.unique(np.nonzero(~np.isfinite(got))[1])
+    np.testing.assert_array_equal(hit, np.unique(np.nonzero(~np.isfinite(other))[1]))
+    assert set(ks) <= set(hit.tolist()) and len(hit) <= 4 * len(ks)
+    rest = np.setdiff1d(np.arange(K), hit)
+    np.testing.assert_array_equal(got[:, rest], clean[:, rest])
+    P.dg_sync_check(s.op)
+    s.close()

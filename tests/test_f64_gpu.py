@@ -179,3 +179,51 @@ def test_small_components_keep_their_precision(P, kind, N, form):
     s.close()
     assert (np.abs(got - want) <= 32 * 2.0 ** -53 * size).all(), \
         float((np.abs(got - want)[size > 0] / size[size > 0]).max() * 2 ** 53)
+
+
+def _solver_and_oracle(P, N, form):
+    mesh = jittered_delaunay_mesh(5, seed=3)
+    d = O.Discretization(*mesh, N)
+    eps = random_permittivity(d.K, seed=2) if form == "media" else None
+    s = P.Solver(*mesh, N=N, precision="fp64", eps=eps)
+    if form == "alpha":
+        P.dg_operator_set_alpha(s.op, 0.25)
+        return d, s, lambda u: O.maxwell_rhs(d, u, alpha=0.25)
+    return d, s, lambda u: O.maxwell_rhs_media(d, u, eps)
+
+
+# the products in FP64 with the second flux scalar and with a permittivity
+@pytest.mark.parametrize("form", ["alpha", "media"])
+@pytest.mark.parametrize("N", range(1, 8))
+@pytest.mark.parametrize("scale", [1e-300, 1e285])
+def test_fp64_products_in_the_other_flux_forms(P, N, form, scale):
+    d, s, rhs = _solver_and_oracle(P, N, form)
+    q = np.random.default_rng(N).uniform(-1, 1, (3, d.K, d.Np))
+    _close(_rhs(P, s, scale * q) / scale, rhs(q))
+    part = q.copy()
+    part[:, : d.K // 2] *= 1e-300
+    _close(_rhs(P, s, part), rhs(part))
+    dt = s.cfl_dt()
+    f, res = s.from_numpy(scale * q), s.new_fields()
+    s.step(f, res, dt, 1)
+    _close(s.to_numpy(f) / scale, O.lsrk_step(d, q, 0.0, dt, rhs=lambda u, t: rhs(u)))
+    s.close()
+
+
+@pytest.mark.parametrize("form", ["alpha", "media"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("N", [1, 4, 7])
+@pytest.mark.parametrize("field", [0, 2])
+def test_non_finite_values_in_the_other_flux_forms(P, N, form, bad, field):
+    d, s, _ = _solver_and_oracle(P, N, form)
+    q = np.random.default_rng(N).uniform(-1, 1, (3, d.K, d.Np))
+    clean = _rhs(P, s, q)
+    k = d.K // 2
+    q[field, k, 0] = bad
+    got = _rhs(P, s, q)
+    reach = {k} | {int(d.EToE[k, f]) for f in range(3)}
+    hit = set(np.nonzero(~np.isfinite(got))[1].tolist())
+    assert k in hit and hit <= reach
+    rest = np.setdiff1d(np.arange(d.K), sorted(reach))
+    np.testing.assert_array_equal(got[:, rest], clean[:, rest])
+    s.close()
