@@ -832,7 +832,7 @@ int32_t dg_test_result_state(int32_t cuda_error);
  * warp first waits, bounded by 0.1 s, for a device flag that nothing sets.
  * The wait runs out, the CTAs set the operator's status word, stop their
  * other warps through their shared abort flag, free their tensor memory and
- * return, having read and written no field.  Synchronises `stream`.  A
+ * return, having written no field.  Synchronises `stream`.  A
  * following dg_sync_check returns DG_ERR_TIMEOUT (and clears the word); the
  * operator stays usable.  The paper has no counterpart: this tests the
  * failure detection of the bounded waits.

@@ -462,9 +462,9 @@ __global__ void __launch_bounds__(Layout<N, MEDIA, E_>::THREADS)
         p.qout[p.fstride + g] = hy + p.b * n1;
         p.qout[2 * p.fstride + g] = ez + p.b * n2;
       }
-      // the operator's point source, on what this thread has just written
-      // (kept out of the update itself, where it held registers: FP64 at
-      // N = 5 ran 1.5 % slower)
+      // the operator's point source, on what this thread has just written: a
+      // branch of its own, so that the update of all other elements holds no
+      // registers for it
       if (k0 + e == p.psrc_k) {
         const float w = p.psrc_w[i];
         if (MODE == kModeRhs) {

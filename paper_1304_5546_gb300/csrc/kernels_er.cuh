@@ -33,13 +33,13 @@
 //
 // Block: 128 elements, a full MMA tile.  Warp roles: two groups of 4 element
 // warps that take blocks in turn (operands into tensor memory; then the
-// accumulators back, chain rule, update in place in the stage buffers), 7 or
-// 10 flux warps (traces element-major, so that a warp's loads coalesce, from
-// the stage where the neighbour is in the block; flux scalars into an array in
-// shared memory), one MMA warp, one memory warp (1D TMA bulk loads into rings
-// of q and geometry stages and of residual stages, bulk stores from both).  Every wait is bounded; on expiry the CTA
-// sets the status word, drains its copies (bounded), frees its TMEM and
-// returns.
+// accumulators back, chain rule, update in place in the stage buffers), 7 flux
+// warps in one group, at N = 3 two groups of 5 (traces element-major, so that a
+// warp's loads coalesce, from the stage where the neighbour is in the block;
+// flux scalars into an array in shared memory), one MMA warp, one memory warp
+// (1D TMA bulk loads into rings of q and geometry stages and of residual
+// stages, bulk stores from both).  Every wait is bounded; on expiry the CTA sets
+// the status word, drains its copies (bounded), frees its TMEM and returns.
 #pragma once
 
 #include <type_traits>
@@ -384,7 +384,8 @@ __global__ void __launch_bounds__(ErLayout<N, MEDIA>::THREADS, 1)
       }
     }
   } else if (warp >= L::FLUX_WARP0) {
-    // ======================= flux warps: two groups that take blocks in turn;
+    // ======================= flux warps, in FLUX_GROUPS groups that take blocks
+    // in turn (one from N = 4 on: every block);
     // thread = face node jn of elements e0, e0 + PER, ... (U of them).  A
     // block's traces are asked for before its stage has landed, from face
     // codes that came straight from global memory a block of the group

@@ -69,12 +69,16 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // launch_chained): wait returns once every kernel this launch depends on has
 // completed and its writes are visible; until then nothing that such a
 // kernel writes may be read, and nothing that it reads may be written.
+// That is griddepcontrol.wait's own guarantee (the memory operations of the
+// grids it waits for are performed and made visible to the waiting grid), and
+// every load behind it rests on it, loads that allocate in L1 among them: the
+// FP64 kernel's fields and residual (written in place, in blocks that share
+// 32-byte sectors with their neighbours'), the traces, and the outputs that a
+// point source reads back.  The read-only path (ld.global.nc, __ldg) is
+// outside of it: it is used for what no launch of a chain writes.
 // trigger lets the next launch of the chain start its own prologue (without
 // it that launch starts as this one's last block ends).  It is called after
-// wait only, so at most two launches of a chain are resident at a time, and
-// by the time a launch starts, the one before its predecessor has ended: no
-// line that the L1 of an SM holds of that launch's input (the buffer its
-// predecessor writes) can be filled after the launch began.
+// wait only, so at most two launches of a chain are resident at a time.
 __device__ __forceinline__ void chain_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
