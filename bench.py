@@ -682,8 +682,7 @@ def run_longrun_study(args):
     (started before any CUDA call); every FP32 variant runs on the GPU from
     the same start.  At each snapshot step: max nodal error relative to
     max |q| of the oracle, and L2 (rms) error relative to the oracle's rms.
-    One JSON line; writes gpurun_out/longrun_gpu_done once the GPU part is
-    over (the oracle may still be running)."""
+    One JSON line."""
     import multiprocessing as mp
 
     import numpy as np
@@ -741,8 +740,6 @@ def run_longrun_study(args):
             gpu[v] = (snaps, ms / c["steps"])
             s.close()
         results.append((c, gpu, dt))
-    os.makedirs(os.path.join(ROOT, "gpurun_out"), exist_ok=True)
-    open(os.path.join(ROOT, "gpurun_out", "longrun_gpu_done"), "w").write("done\n")
     out = []
     for (c, gpu, dt), (pr, conn) in zip(results, workers):
         rows = {v: {"steps": [], "max_rel": [], "l2_rel": []} for v in c["variants"]}
