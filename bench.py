@@ -373,7 +373,9 @@ def run_ours(args):
         return None
 
     K = s.K
-    kernel_kind = s.kernel()[0]
+    kernel_kind, block = s.kernel()
+    family = "f64" if args.precision == "fp64" else "er" if block == 128 else {
+        "tensor cores": "tc", "cuda cores": "simt", "element threads": "ept"}[kernel_kind]
     value = replica_throughput(world, K, args.steps, ms)
     peaks, peak_kind = measured_peaks()
     bytes_step = K * step_bytes_per_element(N) * (2 if args.precision == "fp64" else 1)
@@ -385,8 +387,8 @@ def run_ours(args):
             from paper_1304_5546_gb300.build import kernel_source_hash
             t = json.load(open(tpath))
             key = "N%d_%s" % (N, args.precision)
-            fam = t.get("kernel_family")
-            if t.get("kernel_hash") == kernel_source_hash(fam) and key in t.get("per_element", {}):
+            if (t.get("kernel_family") == family and key in t.get("per_element", {})
+                    and t.get("kernel_hash") == kernel_source_hash(family)):
                 traffic = t["per_element"][key] * K * 5 * args.steps / launches
         except Exception:
             traffic = None
@@ -425,9 +427,7 @@ def run_ours(args):
             "frac": achieved / peaks["hbm_gbs"],
             "traffic": traffic,
             "peak_kind": peak_kind,
-            "kernel": {"tensor cores": "dg_stage_er_kernel" if s.kernel()[1] == 128
-                       else "dg_stage_tc_kernel", "cuda cores": "dg_stage_kernel",
-                       "element threads": "dg_stage_ept_kernel"}[kernel_kind]
+            "kernel": ("dg_stage_kernel" if family == "simt" else "dg_stage_%s_kernel" % family)
                       + " (fused RHS + LSRK stage)",
             "bytes_per_element_step": step_bytes_per_element(N),
         },

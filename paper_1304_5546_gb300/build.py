@@ -92,11 +92,13 @@ def build(force=False, verbose=False, extra_flags=(), checked=False):
 
 
 # Source files that define each stage-kernel family (kernel_source_hash)
+_SHARED = ("kernels.cuh", "launch.h", "ptx.cuh")
 KERNEL_FAMILIES = {
-    "tc": lambda n: (n.startswith("kernels_tc") or n == "kernels.cuh"
-                     or n in ("launch.h", "ptx.cuh")),
-    "ept": lambda n: (n.startswith("kernels_ept") or n == "kernels.cuh"
-                      or n in ("launch.h", "ptx.cuh")),
+    "tc": lambda n: n.startswith("kernels_tc") or n in _SHARED,
+    "er": lambda n: n.startswith("kernels_er") or n == "kernels_tc.cuh" or n in _SHARED,
+    "ept": lambda n: n.startswith("kernels_ept") or n in _SHARED,
+    "f64": lambda n: n.startswith("kernels_f64") or n in _SHARED,
+    "simt": lambda n: n.startswith("kernels_N") or n in _SHARED,
 }
 
 
@@ -105,7 +107,8 @@ def kernel_source_hash(family=None):
     blanks and empty lines are left out); profiles record it so that stale
     counter captures are not reported for a changed kernel.  family: only
     the files of one stage-kernel family (KERNEL_FAMILIES: the tensor-core
-    kernel "tc", the element-thread kernel "ept"); None: every kernel
+    kernel "tc", the element-row kernel "er", the element-thread kernel "ept",
+    the FP64 kernel "f64", the node-thread kernel "simt"); None: every kernel
     source."""
     import hashlib
     import re
