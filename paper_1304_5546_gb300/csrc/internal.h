@@ -128,7 +128,7 @@ struct dg_op {
   void* d_qtmp = nullptr;  // second field buffer for the stage ping-pong
   int* d_flag = nullptr;   // finiteness scan result
   int* d_status = nullptr; // kernel status word (bounded-wait expiry)
-  void* d_tcop = nullptr;  // tensor-core operator tiles for FP32 (see tc_operator_tiles)
+  void* d_tcop = nullptr;  // FP32: tensor-core operator tiles (tc_operator_tiles); FP64: f64_operator_table
   // FP32 on the element-row kernel: what its setup chose (use_er), unless a
   // block size of the other tensor-core kernel was asked for, or
   // dg_operator_tune chose that (er_off); its operator tiles and

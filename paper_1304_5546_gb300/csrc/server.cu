@@ -15,8 +15,8 @@
 //      one dg_batch_step, so requests that arrive while others run join at
 //      the next chunk boundary and share its launches;
 //   4. retires requests that reached their final time: their fields go to
-//      host memory asynchronously (through pinned buffers), their pool
-//      range is freed for the next admission.
+//      host memory asynchronously (by a kernel, or through pinned buffers),
+//      their pool range is freed for the next admission.
 // The host runs at most kAhead chunks ahead of the device.  Each request
 // keeps its own time step (dg_solve's rule: ceil(T / dt_cfl) steps, landing
 // on T) and its own source clock, so its result does not depend on what

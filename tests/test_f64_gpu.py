@@ -8,7 +8,7 @@ import numpy as np
 import pytest
 
 import oracle as O
-from synth import jittered_delaunay_mesh, random_permittivity, square_grid_mesh
+from synth import jittered_delaunay_mesh, random_permittivity
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-12
@@ -158,6 +158,7 @@ def _rhs_and_size(P, s, q, alpha, eps):
 @pytest.mark.parametrize("N", range(1, 8))
 @pytest.mark.parametrize("kind", ["bubbles", "one large"])
 def test_small_components_keep_their_precision(P, kind, N, form):
+    from synth import square_grid_mesh
     mesh = jittered_delaunay_mesh(6, seed=4) if kind == "bubbles" else square_grid_mesh(5, 5)
     s = P.Solver(*mesh, N=N, precision="fp64",
                  eps=random_permittivity(mesh[2].shape[0], seed=2) if form == "media" else None)
